@@ -89,6 +89,7 @@ template <typename T> cudaError_t hmalloc(T **p, size_t bytes) {
 }
 
 constexpr int kGraphSteps = 64;   // even: a replay returns to the same buffer
+constexpr int kObsSlots = kGraphSteps + 2;   // steps of the longest observed chunk
 constexpr int kMaxPalette = 65535;
 
 size_t elem_size(int prec) {
@@ -108,6 +109,7 @@ struct lbm_domain {
   int nx = 0, ny = 0, nxp = 0;
   long long plane = 0;
   size_t esize = 4;
+  int pair_rows = 2;           // row chunk of the two-step kernel
   cudaStream_t stream = nullptr;
   bool own_stream = false;
   void *pop[2] = {nullptr, nullptr};
@@ -140,14 +142,15 @@ struct lbm_domain {
   double bref_next[3] = {0, 0, 0};   // reference b the next reset will use
   cudaGraphExec_t graph[2] = {nullptr, nullptr};
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
-  // observed stepping: per-step (J, heat) sums in device slots [2][64][2],
-  // copied every step into pinned host slots of the same shape; one graph
-  // per (starting buffer, slot half)
-  double *dobs = nullptr, *hobs = nullptr;
+  // observed stepping: the O2 each reacting cell consumes in every step of a
+  // chunk [kObsSlots][reacting rows][nx] (arithmetic precision), its column
+  // sums, the per-step (J, heat) sums in device slots [2][kObsSlots][2], and
+  // pinned host slots of the same shape; one graph per (starting buffer,
+  // slot half)
+  void *jcells = nullptr;
+  double *jcol = nullptr, *dobs = nullptr, *hobs = nullptr;
   cudaGraphExec_t obs_graph[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};
   cudaEvent_t obs_done[2] = {nullptr, nullptr};
-  cudaStream_t obs_side = nullptr;             // the reductions, beside the steps
-  cudaEvent_t obs_fork = nullptr, obs_join = nullptr;
   // x-slab of a larger lattice: columns [x0, x0 + nx) of nxg; a side that
   // borders a neighbour slab reads the ghost column the exchange fills
   int x0 = 0, nxg = 0;
@@ -186,6 +189,11 @@ KArgs make_args(const lbm_domain *d) {
   a.halo_hi = d->halo_hi;
   a.wall_dir = p.wall_dirichlet;
   a.npal = d->npal;
+  a.pair_rows = d->pair_rows;
+  // rows that the two-step kernel asks the L2 cache for ahead of use: only
+  // where the two states do not stay in it from pass to pass (1024 x 256 FP32:
+  // 9.6 us a step without, 10.2 with; 4096 x 1024: 85.8 without, 81.3 with)
+  a.pair_ahead = 48.0 * d->plane * d->esize > 96e6 ? 3 : 0;
   for (int k = 0; k < 3; ++k)
     for (int s = 0; s < 3; ++s) a.Cwall[k][s] = p.C_wall[k][s];
   a.u_in_avg = p.inlet_mode == 0 ? p.u_in_avg : 0.0;
@@ -263,30 +271,82 @@ void drop_graphs(lbm_domain *d) {
       }
 }
 
-lbm_status launch_steps(lbm_domain *d, int64_t n) {
-  const KArgs a = make_args(d);
+// Whether two steps of a domain may run as one launch (k_step2): whole
+// lattices with walls or an inlet and an outlet at the x ends, in the
+// storage types whose step is bound by memory (the FP64 step is bound by its
+// arithmetic), with planes that 32-bit byte offsets reach.  A slab needs its
+// halo between the steps.  Stochastic rounding issues too much for the pair to
+// gain (8192 x 2048 grains, FP16: 510 us a step in pairs, 497 one by one).
+bool can_pair(const lbm_domain *d) {
+  return !fp64(d) && d->desc.rounding == 0 && !d->desc.periodic_x && d->nx == d->nxg &&
+         d->plane * 4 * (long long)d->esize < (1LL << 32);
+}
+
+// How n steps are launched: pairs of steps, then single steps.  A run that
+// ends with a single step (`open` false) leaves the state before its last
+// step in the other buffer, where the read-outs of that step look for it.
+struct StepPlan {
+  int64_t pairs, singles;
+  int64_t launches() const { return pairs + singles; }
+};
+StepPlan plan_steps(const lbm_domain *d, int64_t n, bool open) {
+  StepPlan p{0, n};
+  if (can_pair(d)) {
+    p.pairs = open ? n / 2 : (n > 0 ? (n - 1) / 2 : 0);
+    p.singles = n - 2 * p.pairs;
+  }
+  return p;
+}
+
+// The launches of a plan on stream st, from buffer cur of d on; the j-th
+// step's reaction goes to jout + j jstep elements when jout is not NULL.
+lbm_status launch_plan(lbm_domain *d, const KArgs &a, StepPlan plan, int cur, int variant,
+                       void *jout, int64_t jstep, cudaStream_t st) {
   const DevGeom g = geom(d);
-  for (int64_t k = 0; k < n; ++k) {
+  const size_t rsize = fp64(d) ? 8 : 4;
+  auto slot = [&](int64_t step) {
+    return jout ? (void *)((char *)jout + (size_t)(step * jstep) * rsize) : nullptr;
+  };
+  int64_t step = 0;
+  for (int64_t k = 0; k < plan.launches(); ++k) {
+    const bool pair = k < plan.pairs;
     dispatch(d->desc.precision, [&](auto *tag) {
       using S = std::remove_pointer_t<decltype(tag)>;
-      launch_step<S>(d->pop[d->cur], d->pop[d->cur ^ 1], g, a, d->variant, d->stream);
+      if (pair)
+        launch_step2<S>(d->pop[cur], d->pop[cur ^ 1], g, a, slot(step), jstep, st);
+      else
+        launch_step<S>(d->pop[cur], d->pop[cur ^ 1], g, a, variant, slot(step), st);
     });
-    if (a.stochastic) launch_seed_advance(d->dseed, d->stream);
-    d->cur ^= 1;
+    if (a.stochastic) launch_seed_advance(d->dseed, pair ? 2 : 1, st);
+    step += pair ? 2 : 1;
+    cur ^= 1;
   }
   CK(cudaGetLastError());
   return LBM_OK;
 }
 
+lbm_status launch_steps(lbm_domain *d, int64_t n, bool open = false, void *jout = nullptr,
+                        int64_t jstep = 0) {
+  const StepPlan plan = plan_steps(d, n, open);
+  lbm_status s = launch_plan(d, make_args(d), plan, d->cur, d->variant, jout, jstep, d->stream);
+  if (s == LBM_OK) d->cur ^= (int)(plan.launches() & 1);
+  return s;
+}
+
+// The graph of kGraphSteps steps from the current buffer (an even number of
+// launches either way: a replay ends in the buffer it started from).
 lbm_status ensure_graph(lbm_domain *d) {
   if (d->graph[d->cur]) return LBM_OK;
   const int start = d->cur;
   cudaGraph_t gr = nullptr;
   CK(cudaStreamBeginCapture(d->stream, cudaStreamCaptureModeThreadLocal));
-  lbm_status s = launch_steps(d, kGraphSteps);
+  lbm_status s = launch_steps(d, kGraphSteps, true);
   cudaError_t e = cudaStreamEndCapture(d->stream, &gr);
   d->cur = start;
-  if (s != LBM_OK) return s;
+  if (s != LBM_OK) {
+    if (gr) cudaGraphDestroy(gr);
+    return s;
+  }
   if (e != cudaSuccess) return fail(LBM_ECUDA, "graph capture: %s", cudaGetErrorString(e));
   e = cudaGraphInstantiate(&d->graph[start], gr, 0);
   cudaGraphDestroy(gr);
@@ -294,32 +354,19 @@ lbm_status ensure_graph(lbm_domain *d) {
   return LBM_OK;
 }
 
-// Observed steps: n steps (n <= kGraphSteps).  The reaction of a step is a
-// function of the state it starts from, so its catalyst reduction (into
-// device slot half `half`) and the asynchronous copy of its (J, heat) sums
-// to the pinned host slots run on the side stream concurrently with the
-// step itself; the next step, which overwrites that state, waits for them.
-lbm_status launch_observed(lbm_domain *d, int64_t n, int half) {
+// Observed steps: n steps (n <= kObsSlots) that also write the O2 every
+// reacting cell consumes, [step][reacting row][nx], then the FP64 sums of
+// every step and their copy to the pinned host slots of `half`.
+lbm_status launch_observed(lbm_domain *d, int64_t n, bool open, int half) {
+  const int64_t rows = d->desc.reaction_mode == 1 ? d->desc.ny_cl : 1;
+  lbm_status s = launch_steps(d, n, open, d->jcells, rows * d->nx);
+  if (s != LBM_OK) return s;
   const KArgs a = make_args(d);
-  const lbm_params &p = d->prm;
-  const double i_scale = 4.0 * p.F * p.c_tot * p.dx_cm / p.dt_s;
-  for (int64_t k = 0; k < n; ++k) {
-    if (k > 0) CK(cudaStreamWaitEvent(d->stream, d->obs_join, 0));
-    CK(cudaEventRecord(d->obs_fork, d->stream));
-    CK(cudaStreamWaitEvent(d->obs_side, d->obs_fork, 0));
-    const size_t slot = ((size_t)half * kGraphSteps + (size_t)k) * 2;
-    dispatch(d->desc.precision, [&](auto *tag) {
-      using S = std::remove_pointer_t<decltype(tag)>;
-      launch_catalyst<S>(d->pop[d->cur], geom(d), a, i_scale, nullptr, d->colsum,
-                         d->dobs + slot, d->obs_side);
-    });
-    CK(cudaMemcpyAsync(d->hobs + slot, d->dobs + slot, 2 * sizeof(double),
-                       cudaMemcpyDeviceToHost, d->obs_side));
-    CK(cudaEventRecord(d->obs_join, d->obs_side));
-    lbm_status s = launch_steps(d, 1);
-    if (s != LBM_OK) return s;
-  }
-  if (n > 0) CK(cudaStreamWaitEvent(d->stream, d->obs_join, 0));
+  const size_t slot = (size_t)half * kObsSlots * 2;
+  launch_sum_reaction(d->jcells, fp64(d), d->nx, (int)rows, (int)n, a.hpo, d->jcol, d->dobs + slot,
+                      d->stream);
+  CK(cudaMemcpyAsync(d->hobs + slot, d->dobs + slot, (size_t)n * 2 * sizeof(double),
+                     cudaMemcpyDeviceToHost, d->stream));
   CK(cudaGetLastError());
   return LBM_OK;
 }
@@ -330,14 +377,50 @@ lbm_status ensure_obs_graph(lbm_domain *d, int half) {
   const int start = d->cur;
   cudaGraph_t gr = nullptr;
   CK(cudaStreamBeginCapture(d->stream, cudaStreamCaptureModeThreadLocal));
-  lbm_status s = launch_observed(d, kGraphSteps, half);
+  lbm_status s = launch_observed(d, kGraphSteps, true, half);
   cudaError_t e = cudaStreamEndCapture(d->stream, &gr);
   d->cur = start;
-  if (s != LBM_OK) return s;
+  if (s != LBM_OK) {
+    if (gr) cudaGraphDestroy(gr);
+    return s;
+  }
   if (e != cudaSuccess) return fail(LBM_ECUDA, "graph capture: %s", cudaGetErrorString(e));
-  e = cudaGraphInstantiateWithFlags(&ge, gr, cudaGraphInstantiateFlagUseNodePriority);
+  e = cudaGraphInstantiate(&ge, gr, 0);
   cudaGraphDestroy(gr);
   if (e != cudaSuccess) return fail(LBM_ECUDA, "graph instantiate: %s", cudaGetErrorString(e));
+  return LBM_OK;
+}
+
+// First-use work space of observed stepping, all or nothing.
+lbm_status ensure_observation(lbm_domain *d) {
+  if (d->dobs) return LBM_OK;
+  const size_t bytes = 2 * kObsSlots * 2 * sizeof(double);
+  const size_t rows = d->desc.reaction_mode == 1 ? d->desc.ny_cl : 1;
+  const size_t jbytes = (size_t)kObsSlots * rows * d->nx * (fp64(d) ? 8 : 4);
+  double *dobs = nullptr, *hobs = nullptr, *jcol = nullptr;
+  void *jcells = nullptr;
+  cudaEvent_t done[2] = {nullptr, nullptr};
+  if (dmalloc(&dobs, bytes) != cudaSuccess || hmalloc(&hobs, bytes) != cudaSuccess ||
+      dmalloc(&jcol, sizeof(double) * 2 * kObsSlots * d->nx) != cudaSuccess ||
+      dmalloc(&jcells, jbytes) != cudaSuccess ||
+      cudaEventCreateWithFlags(&done[0], cudaEventDisableTiming) != cudaSuccess ||
+      cudaEventCreateWithFlags(&done[1], cudaEventDisableTiming) != cudaSuccess ||
+      // cells that never react (solids) keep their zeros
+      cudaMemsetAsync(jcells, 0, jbytes, d->stream) != cudaSuccess) {
+    for (void *p : {(void *)dobs, (void *)jcol, jcells})
+      if (p) cudaFree(p);
+    if (hobs) cudaFreeHost(hobs);
+    for (cudaEvent_t e : done)
+      if (e) cudaEventDestroy(e);
+    cudaGetLastError();
+    return fail(LBM_ENOMEM, "observation slots (%.1f MB)", jbytes / 1e6);
+  }
+  d->dobs = dobs;
+  d->hobs = hobs;
+  d->jcol = jcol;
+  d->jcells = jcells;
+  d->obs_done[0] = done[0];
+  d->obs_done[1] = done[1];
   return LBM_OK;
 }
 
@@ -450,7 +533,12 @@ lbm_status lbm_create_domain(const lbm_domain_desc *desc, lbm_domain **out) {
   // untuned default: 64 x 2 cells at 8 blocks per SM for FP32 storage (the
   // tuner's usual choice at large sizes), the uncapped 128 x 2 otherwise
   d->variant = D.precision == LBM_FP32 ? 7 : 0;
+  d->pair_rows = pair_rows(&d->nx, &d->ny, &D.ny_cl, 1, d->esize);
   auto cleanup = [&](lbm_status s) { lbm_destroy_domain(d); return s; };
+  cudaError_t allowed = cudaSuccess;
+  dispatch(D.precision, [&](auto *tag) { allowed = allow_step2<std::remove_pointer_t<decltype(tag)>>(); });
+  if (allowed != cudaSuccess)
+    return cleanup(fail(LBM_ECUDA, "shared memory of the two-step kernel: %s", cudaGetErrorString(allowed)));
   if (D.cuda_stream) {
     d->stream = (cudaStream_t)D.cuda_stream;
   } else {
@@ -503,13 +591,13 @@ lbm_status lbm_destroy_domain(lbm_domain *d) {
   drop_graphs(d);
   for (void *p : {d->pop[0], d->pop[1], (void *)d->mask, (void *)d->mid, d->pal, (void *)d->raw,
                   d->snap, (void *)d->partial, (void *)d->colsum, (void *)d->dsmall, (void *)d->dbad, (void *)d->dseed,
-                  (void *)d->scratch, (void *)d->dprofile, (void *)d->dobs, d->pal_scratch})
+                  (void *)d->scratch, (void *)d->dprofile, (void *)d->dobs, d->jcells, (void *)d->jcol,
+                  d->pal_scratch})
     if (p) cudaFree(p);
   if (d->hsmall) cudaFreeHost(d->hsmall);
   if (d->hobs) cudaFreeHost(d->hobs);
-  for (auto e : {d->obs_done[0], d->obs_done[1], d->obs_fork, d->obs_join})
+  for (auto e : {d->obs_done[0], d->obs_done[1]})
     if (e) cudaEventDestroy(e);
-  if (d->obs_side) cudaStreamDestroy(d->obs_side);
   if (d->ev0) cudaEventDestroy(d->ev0);
   if (d->ev1) cudaEventDestroy(d->ev1);
   if (d->ev_halo) cudaEventDestroy(d->ev_halo);
@@ -752,8 +840,9 @@ lbm_status lbm_step(lbm_domain *d, int64_t nsteps) {
   lbm_status s = check_ready(d);
   if (s != LBM_OK) return s;
   if (nsteps < 0) return fail(LBM_EINVAL, "nsteps < 0");
+  // long runs replay a graph; the last step or two are launched on their own
   int64_t left = nsteps;
-  while (left >= 2 * kGraphSteps) {
+  while (left >= 2 * kGraphSteps || (d->graph[d->cur] && left >= kGraphSteps + 2)) {
     if ((s = ensure_graph(d)) != LBM_OK) return s;
     CK(cudaGraphLaunch(d->graph[d->cur], d->stream));
     left -= kGraphSteps;
@@ -806,43 +895,16 @@ lbm_status lbm_step_observe(lbm_domain *d, int64_t nsteps, double *i_avg, double
   if (s != LBM_OK) return s;
   if (nsteps < 0) return fail(LBM_EINVAL, "nsteps < 0");
   if (nsteps > 0 && !i_avg && !heat) return fail(LBM_EINVAL, "nothing to observe (use lbm_step)");
-  if (!d->dobs) {
-    // the reductions run at the highest priority, so that their few blocks
-    // are dispatched while the step's blocks are still being issued
-    // instead of after them
-    int lo_prio = 0, hi_prio = 0;
-    const size_t bytes = 2 * kGraphSteps * 2 * sizeof(double);
-    if (dmalloc(&d->dobs, bytes) != cudaSuccess || hmalloc(&d->hobs, bytes) != cudaSuccess ||
-        cudaDeviceGetStreamPriorityRange(&lo_prio, &hi_prio) != cudaSuccess ||
-        cudaStreamCreateWithPriority(&d->obs_side, cudaStreamNonBlocking, hi_prio) != cudaSuccess ||
-        cudaEventCreateWithFlags(&d->obs_fork, cudaEventDisableTiming) != cudaSuccess ||
-        cudaEventCreateWithFlags(&d->obs_join, cudaEventDisableTiming) != cudaSuccess ||
-        cudaEventCreateWithFlags(&d->obs_done[0], cudaEventDisableTiming) != cudaSuccess ||
-        cudaEventCreateWithFlags(&d->obs_done[1], cudaEventDisableTiming) != cudaSuccess) {
-      // release what was made, so that a later call starts over
-      if (d->dobs) cudaFree(d->dobs);
-      if (d->hobs) cudaFreeHost(d->hobs);
-      if (d->obs_side) cudaStreamDestroy(d->obs_side);
-      for (cudaEvent_t *e : {&d->obs_fork, &d->obs_join, &d->obs_done[0], &d->obs_done[1]})
-        if (*e) {
-          cudaEventDestroy(*e);
-          *e = nullptr;
-        }
-      d->dobs = d->hobs = nullptr;
-      d->obs_side = nullptr;
-      cudaGetLastError();
-      return fail(LBM_ENOMEM, "observation slots");
-    }
-  }
+  if ((s = ensure_observation(d)) != LBM_OK) return s;
   const lbm_params &p = d->prm;
   const double i_scale = 4.0 * p.F * p.c_tot * p.dx_cm / p.dt_s;
   const double q_scale = p.rho_cp_f * p.dx_cm / p.dt_s;
-  // chunks of up to kGraphSteps steps alternate between the two slot halves:
-  // while chunk c runs, the host reads chunk c - 1's slots
+  // chunks alternate between the two slot halves: while one runs, the host
+  // reads the other's slots.  The last chunk ends with a single step.
   auto collect = [&](int half, int64_t first, int64_t n) -> lbm_status {
     CK(cudaEventSynchronize(d->obs_done[half]));
     for (int64_t k = 0; k < n; ++k) {
-      const double *v = d->hobs + ((size_t)half * kGraphSteps + (size_t)k) * 2;
+      const double *v = d->hobs + ((size_t)half * kObsSlots + (size_t)k) * 2;
       if (i_avg) i_avg[first + k] = v[0] * i_scale / d->nx;
       if (heat) heat[first + k] = v[1] * q_scale / d->nx;
     }
@@ -851,11 +913,12 @@ lbm_status lbm_step_observe(lbm_domain *d, int64_t nsteps, double *i_avg, double
   int64_t done = 0, prev_first = -1, prev_n = 0;
   int half = 0;
   while (done < nsteps) {
-    const int64_t n = std::min<int64_t>(kGraphSteps, nsteps - done);
-    if (n == kGraphSteps) {
+    const bool last = nsteps - done <= kObsSlots;
+    const int64_t n = last ? nsteps - done : kGraphSteps;
+    if (!last) {
       if ((s = ensure_obs_graph(d, half)) != LBM_OK) return s;
-      CK(cudaGraphLaunch(d->obs_graph[d->cur][half], d->stream));   // even: cur unchanged
-    } else if ((s = launch_observed(d, n, half)) != LBM_OK) {
+      CK(cudaGraphLaunch(d->obs_graph[d->cur][half], d->stream));   // cur unchanged
+    } else if ((s = launch_observed(d, n, false, half)) != LBM_OK) {
       return s;
     }
     CK(cudaEventRecord(d->obs_done[half], d->stream));
@@ -1070,7 +1133,7 @@ lbm_status lbm_tune(lbm_domain *d, int32_t trial_steps, int32_t *variant, double
         dispatch(d->desc.precision, [&](auto *tag) {
           using S = std::remove_pointer_t<decltype(tag)>;
           // the same step from the same state every time: the state is kept
-          launch_step<S>(d->pop[d->cur], d->pop[d->cur ^ 1], g, a, v, d->stream);
+          launch_step<S>(d->pop[d->cur], d->pop[d->cur ^ 1], g, a, v, nullptr, d->stream);
         });
     };
     run(2);
@@ -1631,6 +1694,12 @@ struct lbm_batch {
   cudaEvent_t ev_fork = nullptr;
   cudaGraphExec_t conc_graph = nullptr;
   std::vector<int> conc_cur;
+  std::vector<int> flips;           // per case: whether the last run ended in the other buffer
+  // schedule 0 in steps of two (every case can_pair): blocks of the two-step
+  // kernel, numbered case after case
+  bool pairs = false;
+  int *dpair = nullptr;             // device prefix sums [ncases + 1]
+  int pair_blocks = 0, pair_rows = 0;
   std::vector<KArgs> conc_args;     // the arguments the graph's launches carry
 };
 
@@ -1650,9 +1719,10 @@ void drop_batch_graph(lbm_batch *b) {
 }
 
 // Schedule 3: n steps of every case, each case on its own lane stream,
-// forked from and joined back into the batch stream.  fixed_parity: every
-// step starts from the case's current state (tuner trials).
-lbm_status batch_lanes(lbm_batch *b, int64_t n, bool fixed_parity) {
+// forked from and joined back into the batch stream.  fixed_parity: n trials
+// of two steps each, every one from the case's current state (tuner).
+// open: the run goes on, it need not end with a single step (plan_steps).
+lbm_status batch_lanes(lbm_batch *b, int64_t n, bool fixed_parity, bool open) {
   const int nc = (int)b->doms.size();
   if ((int)b->lanes.size() != nc) {
     // all or nothing: a partial set is released, so a later call starts over
@@ -1683,13 +1753,15 @@ lbm_status batch_lanes(lbm_batch *b, int64_t n, bool fixed_parity) {
     lbm_domain *d = b->doms[c];
     const KArgs a = make_args(d);
     CK(cudaStreamWaitEvent(b->lanes[c], b->ev_fork, 0));
-    for (int64_t k = 0; k < n; ++k) {
-      const int src = fixed_parity ? d->cur : (int)(d->cur ^ (k & 1));
-      dispatch(b->precision, [&](auto *tag) {
-        using S = std::remove_pointer_t<decltype(tag)>;
-        launch_step<S>(d->pop[src], d->pop[src ^ 1], geom(d), a, b->variant, b->lanes[c]);
-      });
+    // trials: the same launch again and again, two steps' worth each
+    const bool pair = can_pair(d);
+    const int64_t reps = fixed_parity ? (pair ? n : 2 * n) : 1;
+    const StepPlan plan = !fixed_parity ? plan_steps(d, n, open) : pair ? StepPlan{1, 0} : StepPlan{0, 1};
+    for (int64_t k = 0; k < reps; ++k) {
+      lbm_status s = launch_plan(d, a, plan, d->cur, b->variant, nullptr, 0, b->lanes[c]);
+      if (s != LBM_OK) return s;
     }
+    b->flips[c] = (int)(plan.launches() & 1);
     CK(cudaEventRecord(b->lane_done[c], b->lanes[c]));
     CK(cudaStreamWaitEvent(b->stream, b->lane_done[c], 0));
   }
@@ -1732,6 +1804,7 @@ lbm_status batch_table(lbm_batch *b, int bx) {
     bc.pal = d->pal;
     bc.cur0 = d->cur;
     bc.tiles_x = (d->nx + bx - 1) / bx;
+    if (b->pairs) bc.a.pair_rows = b->pair_rows;
   }
   dispatch(b->precision, [&](auto *tag) {
     using S = std::remove_pointer_t<decltype(tag)>;
@@ -1755,19 +1828,27 @@ lbm_status batch_join_out(lbm_batch *b) {
   return LBM_OK;
 }
 
-void batch_launch_steps(lbm_batch *b, int64_t n, int parity0) {
-  for (int64_t k = 0; k < n; ++k)
+// The launches of n steps of schedule 0: all cases alike.
+StepPlan batch_plan(const lbm_batch *b, int64_t n, bool open) {
+  return b->pairs ? plan_steps(b->doms[0], n, open) : StepPlan{0, n};
+}
+void batch_launch_plan(lbm_batch *b, StepPlan plan) {
+  for (int64_t k = 0; k < plan.launches(); ++k)
     dispatch(b->precision, [&](auto *tag) {
       using S = std::remove_pointer_t<decltype(tag)>;
-      launch_batch_step<S>(b->dcases, b->dtile, (int)b->doms.size(), b->total_tiles, b->variant,
-                           (int)((parity0 + k) & 1), b->stream);
+      if (k < plan.pairs)
+        launch_batch_step2<S>(b->dcases, b->dpair, (int)b->doms.size(), b->pair_blocks, (int)(k & 1),
+                              b->stream);
+      else
+        launch_batch_step<S>(b->dcases, b->dtile, (int)b->doms.size(), b->total_tiles, b->variant,
+                             (int)(k & 1), b->stream);
     });
 }
 
 lbm_status batch_run(lbm_batch *b, int64_t nsteps, bool fixed_parity) {
   const int n = (int)b->doms.size();
   if (b->schedule == 3) {              // concurrent chains of single-domain launches
-    if (fixed_parity) return batch_lanes(b, nsteps, true);
+    if (fixed_parity) return batch_lanes(b, nsteps, true, true);
     std::vector<int> cur(n);
     std::vector<KArgs> args(n);
     for (int c = 0; c < n; ++c) {
@@ -1781,13 +1862,16 @@ lbm_status batch_run(lbm_batch *b, int64_t nsteps, bool fixed_parity) {
          std::memcmp(args.data(), b->conc_args.data(), sizeof(KArgs) * n) != 0))
       drop_batch_graph(b);
     int64_t left = nsteps;
-    while (left >= 2 * kBatchGraphSteps) {
+    while (left >= 2 * kBatchGraphSteps || (b->conc_graph && left >= kBatchGraphSteps + 2)) {
       if (!b->conc_graph) {
         cudaGraph_t gr = nullptr;
         CK(cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal));
-        lbm_status s = batch_lanes(b, kBatchGraphSteps, false);
+        lbm_status s = batch_lanes(b, kBatchGraphSteps, false, true);
         cudaError_t e = cudaStreamEndCapture(b->stream, &gr);
-        if (s != LBM_OK) return s;
+        if (s != LBM_OK) {
+          if (gr) cudaGraphDestroy(gr);
+          return s;
+        }
         if (e != cudaSuccess) return fail(LBM_ECUDA, "lane graph capture: %s", cudaGetErrorString(e));
         e = cudaGraphInstantiate(&b->conc_graph, gr, 0);
         cudaGraphDestroy(gr);
@@ -1798,8 +1882,9 @@ lbm_status batch_run(lbm_batch *b, int64_t nsteps, bool fixed_parity) {
       CK(cudaGraphLaunch(b->conc_graph, b->stream));   // even count: parities return
       left -= kBatchGraphSteps;
     }
-    return left > 0 ? batch_lanes(b, left, false) : LBM_OK;
+    return batch_lanes(b, left, false, false);
   }
+  for (int &f : b->flips) f = (int)(nsteps & 1);
   if (b->schedule == 2) {              // one launch per case and step, no graph
     for (int64_t k = 0; k < nsteps; ++k)
       for (lbm_domain *d : b->doms) {
@@ -1807,7 +1892,7 @@ lbm_status batch_run(lbm_batch *b, int64_t nsteps, bool fixed_parity) {
         const int src = fixed_parity ? d->cur : (int)(d->cur ^ (k & 1));
         dispatch(b->precision, [&](auto *tag) {
           using S = std::remove_pointer_t<decltype(tag)>;
-          launch_step<S>(d->pop[src], d->pop[src ^ 1], geom(d), a, d->variant, b->stream);
+          launch_step<S>(d->pop[src], d->pop[src ^ 1], geom(d), a, d->variant, nullptr, b->stream);
         });
       }
     CK(cudaGetLastError());
@@ -1851,32 +1936,36 @@ lbm_status batch_run(lbm_batch *b, int64_t nsteps, bool fixed_parity) {
     }
     return LBM_OK;
   }
-  // schedule 0: one launch per step over all tiles, replayed from a graph
+  // schedule 0: one launch over all tiles per step, or per two steps,
+  // replayed from a graph
   const StepShape sh = kStepShapes[b->variant];
   lbm_status s = batch_tiles(b, sh.bx, sh.by * kBatchRows);
   if (s != LBM_OK) return s;
   if ((s = batch_table(b, sh.bx)) != LBM_OK) return s;
-  if (fixed_parity) {
-    for (int64_t k = 0; k < nsteps; ++k) batch_launch_steps(b, 1, 0);
+  if (fixed_parity) {   // trials of two steps each, as batch_lanes
+    for (int64_t k = 0; k < (b->pairs ? nsteps : 2 * nsteps); ++k)
+      batch_launch_plan(b, b->pairs ? StepPlan{1, 0} : StepPlan{0, 1});
     CK(cudaGetLastError());
     return LBM_OK;
   }
   int64_t left = nsteps;
-  while (left >= 2 * kBatchGraphSteps) {
+  while (left >= 2 * kBatchGraphSteps || (b->graph && left >= kBatchGraphSteps + 2)) {
     if (!b->graph) {
       cudaGraph_t gr = nullptr;
       CK(cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal));
-      batch_launch_steps(b, kBatchGraphSteps, 0);
+      batch_launch_plan(b, batch_plan(b, kBatchGraphSteps, true));
       cudaError_t e = cudaStreamEndCapture(b->stream, &gr);
       if (e != cudaSuccess) return fail(LBM_ECUDA, "batch graph capture: %s", cudaGetErrorString(e));
       e = cudaGraphInstantiate(&b->graph, gr, 0);
       cudaGraphDestroy(gr);
       if (e != cudaSuccess) return fail(LBM_ECUDA, "batch graph instantiate: %s", cudaGetErrorString(e));
     }
-    CK(cudaGraphLaunch(b->graph, b->stream));   // even count: parity returns to 0
+    CK(cudaGraphLaunch(b->graph, b->stream));   // an even number of launches: parity returns to 0
     left -= kBatchGraphSteps;
   }
-  batch_launch_steps(b, left, 0);
+  const StepPlan plan = batch_plan(b, left, false);
+  batch_launch_plan(b, plan);
+  for (int &f : b->flips) f = (int)(plan.launches() & 1);
   CK(cudaGetLastError());
   return LBM_OK;
 }
@@ -1908,14 +1997,32 @@ lbm_status lbm_create_batch(lbm_domain *const *domains, int32_t ncases, lbm_batc
   b->precision = domains[0]->desc.precision;
   b->stream = domains[0]->stream;
   b->ev.resize(ncases, nullptr);
+  b->flips.assign(ncases, 0);
   auto cleanup = [&](lbm_status s) { lbm_destroy_batch(b); return s; };
   if (dmalloc(&b->dcases, sizeof(BatchCase) * ncases) != cudaSuccess ||
       hmalloc(&b->hcases, sizeof(BatchCase) * ncases) != cudaSuccess ||
       dmalloc(&b->dtile, sizeof(int) * (ncases + 1)) != cudaSuccess ||
+      dmalloc(&b->dpair, sizeof(int) * (ncases + 1)) != cudaSuccess ||
       dmalloc(&b->dbar, 2 * sizeof(unsigned)) != cudaSuccess ||
       dmalloc(&b->dstatus, sizeof(int)) != cudaSuccess) {
     cudaGetLastError();
     return cleanup(fail(LBM_ENOMEM, "batch tables"));
+  }
+  b->pairs = true;
+  for (const lbm_domain *d : b->doms) b->pairs = b->pairs && can_pair(d);
+  if (b->pairs) {
+    std::vector<int> nx(ncases), ny(ncases), ny_cl(ncases), start(ncases + 1, 0);
+    for (int c = 0; c < ncases; ++c) {
+      nx[c] = b->doms[c]->nx;
+      ny[c] = b->doms[c]->ny;
+      ny_cl[c] = b->doms[c]->desc.ny_cl;
+    }
+    b->pair_rows = pair_rows(nx.data(), ny.data(), ny_cl.data(), ncases, b->doms[0]->esize);
+    for (int c = 0; c < ncases; ++c)
+      start[c + 1] = start[c] + pair_blocks(nx[c], ny[c], ny_cl[c], b->pair_rows);
+    b->pair_blocks = start[ncases];
+    if (cudaMemcpy(b->dpair, start.data(), sizeof(int) * (ncases + 1), cudaMemcpyHostToDevice) != cudaSuccess)
+      return cleanup(fail(LBM_ECUDA, "batch tables"));
   }
   for (auto &e : b->ev)
     if (cudaEventCreateWithFlags(&e, cudaEventDisableTiming) != cudaSuccess)
@@ -1931,7 +2038,7 @@ lbm_status lbm_destroy_batch(lbm_batch *b) {
   if (!b) return LBM_OK;
   if (b->stream) cudaStreamSynchronize(b->stream);
   drop_batch_graph(b);
-  for (void *p : {(void *)b->dcases, (void *)b->dtile, (void *)b->dbar, (void *)b->dstatus})
+  for (void *p : {(void *)b->dcases, (void *)b->dtile, (void *)b->dpair, (void *)b->dbar, (void *)b->dstatus})
     if (p) cudaFree(p);
   if (b->hcases) cudaFreeHost(b->hcases);
   for (auto e : b->ev)
@@ -1970,8 +2077,8 @@ lbm_status lbm_batch_step(lbm_batch *b, int64_t nsteps) {
   lbm_status s = batch_join_in(b);
   if (s != LBM_OK) return s;
   if ((s = batch_run(b, nsteps, false)) != LBM_OK) return s;
-  for (lbm_domain *d : b->doms) {
-    d->cur ^= (int)(nsteps & 1);
+  for (lbm_domain *&d : b->doms) {
+    d->cur ^= b->flips[&d - b->doms.data()];
     d->steps += nsteps;
   }
   return batch_join_out(b);
@@ -2017,8 +2124,10 @@ lbm_status lbm_batch_tune(lbm_batch *b, int32_t trial_steps, int32_t *schedule, 
     CK(cudaEventSynchronize(b->ev1));
     float ms = 0;
     CK(cudaEventElapsedTime(&ms, b->ev0, b->ev1));
-    if (ms / trial_steps < best) {
-      best = ms / trial_steps;
+    // (the persistent schedule tries single steps, the others two at a time)
+    const double per_step = ms / trial_steps / (sched == 1 ? 1 : 2);
+    if (per_step < best) {
+      best = per_step;
       best_sched = sched;
       best_var = var;
     }

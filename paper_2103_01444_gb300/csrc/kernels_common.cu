@@ -80,9 +80,42 @@ __global__ void k_halo_copy(const S *__restrict__ src, long long src_plane, int 
   dst[di] = src[si];
 }
 
-__global__ void k_seed_advance(unsigned *ctr) { *ctr += 1u; }
+__global__ void k_seed_advance(unsigned *ctr, unsigned n) { *ctr += n; }
 
-void launch_seed_advance(unsigned *ctr, cudaStream_t st) { k_seed_advance<<<1, 1, 0, st>>>(ctr); }
+void launch_seed_advance(unsigned *ctr, unsigned n, cudaStream_t st) {
+  k_seed_advance<<<1, 1, 0, st>>>(ctr, n);
+}
+
+// The row chunk of the two-step kernel's warps.  A unit of h weighted rows (a
+// catalyst row counts two) takes h + 2 first and h second steps of a row, and
+// about four row steps pass before its first row has arrived.  Units are
+// uneven (the end columns cost more), so with more of them than fit the GPU
+// at once the time is their total over the slots plus most of one unit, and
+// with fewer twice an even unit's.  Measured, FP32, us a step: 4096 x 1024 at
+// 8 / 12 / 16 / 24 / 32 / 48 rows 88 / 83 / 81 / 85 / 94 / 122 (the rule
+// takes 16); 1024 x 256 at 1 / 2 / 3 / 4 / 8 rows 11.4 / 9.6 / 9.7 / 10.2 /
+// 14.9 (3); 200 x 40 at 1 / 2 / 8 rows 3.6 / 4.7 / 11.9 (1).
+static long long pair_units(int nx, int ny, int ny_cl, int rows) {
+  return (long long)((nx + kStripCols - 1) / kStripCols) * ((ny + ny_cl + rows - 1) / rows);
+}
+int pair_blocks(int nx, int ny, int ny_cl, int rows) {
+  return (int)((pair_units(nx, ny, ny_cl, rows) + kPairWarps - 1) / kPairWarps);
+}
+int pair_rows(const int *nx, const int *ny, const int *ny_cl, int n, size_t esize) {
+  const double slots = 152.0 * kPairWarps * pair_blocks_per_sm(esize);
+  double best = 1e300;
+  int rows = 1;
+  for (int h = 1; h <= 64; ++h) {
+    double units = 0;
+    for (int k = 0; k < n; ++k) units += (double)pair_units(nx[k], ny[k], ny_cl[k], h);
+    const double waves = units / slots, cost = (waves <= 1.0 ? 2.0 : waves + 0.8) * (2 * h + 6);
+    if (cost < best) {
+      best = cost;
+      rows = h;
+    }
+  }
+  return rows;
+}
 
 void launch_build_mask(uint8_t *mask, const uint8_t *solid, int nx, int ny, int nxp, int ny_cl,
                        int ny_gdl, int mode, int periodic, int closed, int x0, int nxg,
@@ -175,6 +208,8 @@ __global__ void __launch_bounds__(kReduceThreads)
 k_sum_columns(const double *__restrict__ colsum, int nx, double *__restrict__ out) {
   __shared__ double sm[2 * 32];
   double acc[2] = {0.0, 0.0};
+  colsum += (long long)blockIdx.x * 2 * nx;
+  out += 2 * blockIdx.x;
   for (int x = threadIdx.x; x < nx; x += blockDim.x) {
     acc[0] += colsum[x];
     acc[1] += colsum[nx + x];
@@ -184,6 +219,18 @@ k_sum_columns(const double *__restrict__ colsum, int nx, double *__restrict__ ou
     out[0] = acc[0];
     out[1] = acc[1];
   }
+}
+
+void launch_sum_reaction(const void *jcells, bool fp64, int nx, int rows, int nsteps, double hpo,
+                         double *colsum, double *out, cudaStream_t st) {
+  const dim3 grid((nx + kCatalystBX - 1) / kCatalystBX, nsteps);
+  if (fp64)
+    k_sum_cells<double><<<grid, kCatalystBX * kCatalystBY, 0, st>>>((const double *)jcells, nx, rows,
+                                                                    hpo, colsum);
+  else
+    k_sum_cells<float><<<grid, kCatalystBX * kCatalystBY, 0, st>>>((const float *)jcells, nx, rows,
+                                                                   hpo, colsum);
+  k_sum_columns<<<nsteps, kReduceThreads, 0, st>>>(colsum, nx, out);
 }
 
 }  // namespace pemlbm

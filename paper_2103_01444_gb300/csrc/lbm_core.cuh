@@ -71,6 +71,10 @@ enum : uint8_t {
 };
 
 // --------------------------------------------------------------- storage
+// Where a kernel reads populations from: a global buffer through the
+// read-only path, a global buffer past L1, or the row ring that the
+// two-step kernel keeps in shared memory (Pops).
+enum : int { kLdg = 0, kLdcg = 1, kRing = 2 };
 template <typename S> struct Real { using type = float; };
 template <> struct Real<double> { using type = double; };
 
@@ -96,10 +100,17 @@ __device__ __forceinline__ float ld_cg(const __half *p) {
   const unsigned short b = __ldcg(reinterpret_cast<const unsigned short *>(p));
   return __half2float(__ushort_as_half(b));
 }
-template <bool CG, typename S> __device__ __forceinline__ auto ldp(const S *p) {
-  if constexpr (CG) return ld_cg(p);
+template <int CG, typename S> __device__ __forceinline__ auto ldp(const S *p) {
+  if constexpr (CG == kLdcg) return ld_cg(p);
   else return ld_r(p);
 }
+
+// Plain loads, for shared memory.
+__device__ __forceinline__ float ld_s(const float *p) { return *p; }
+__device__ __forceinline__ float ld_s(const __nv_bfloat16 *p) {
+  return __uint_as_float((unsigned)*reinterpret_cast<const unsigned short *>(p) << 16);
+}
+__device__ __forceinline__ float ld_s(const __half *p) { return __half2float(*p); }
 
 // Stochastic rounding of a step's 16-bit stores: unbiased, E[stored] = v,
 // so increments far below half an ulp of a stored value still accumulate.
@@ -143,31 +154,48 @@ __device__ __forceinline__ unsigned xorshift32(unsigned &s) {
 
 // One group of four values (links i of the flow and of the three scalars).
 template <typename R> struct Quad { R v[4]; };
-template <bool CG>
+template <int CG>
 __device__ __forceinline__ Quad<float> ldq(const float *p) {
   const float4 *q = reinterpret_cast<const float4 *>(p);
-  const float4 t = CG ? __ldcg(q) : __ldg(q);
+  const float4 t = CG == kLdcg ? __ldcg(q) : __ldg(q);
   return Quad<float>{{t.x, t.y, t.z, t.w}};
 }
-template <bool CG>
+template <int CG>
 __device__ __forceinline__ Quad<double> ldq(const double *p) {
   const double2 *q = reinterpret_cast<const double2 *>(p);
-  const double2 t0 = CG ? __ldcg(q) : __ldg(q), t1 = CG ? __ldcg(q + 1) : __ldg(q + 1);
+  const double2 t0 = CG == kLdcg ? __ldcg(q) : __ldg(q), t1 = CG == kLdcg ? __ldcg(q + 1) : __ldg(q + 1);
   return Quad<double>{{t0.x, t0.y, t1.x, t1.y}};
 }
 // 16-bit groups: one 8-byte load, the first value in the low half of the
 // first word; each conversion is exact (as __bfloat162float, __half2float)
-template <bool CG>
+template <int CG>
 __device__ __forceinline__ Quad<float> ldq(const __nv_bfloat16 *p) {
   const uint2 *q = reinterpret_cast<const uint2 *>(p);
-  const uint2 t = CG ? __ldcg(q) : __ldg(q);
+  const uint2 t = CG == kLdcg ? __ldcg(q) : __ldg(q);
   return Quad<float>{{__uint_as_float(t.x << 16), __uint_as_float(t.x & 0xffff0000u),
                       __uint_as_float(t.y << 16), __uint_as_float(t.y & 0xffff0000u)}};
 }
-template <bool CG>
+template <int CG>
 __device__ __forceinline__ Quad<float> ldq(const __half *p) {
   const uint2 *q = reinterpret_cast<const uint2 *>(p);
-  const uint2 t = CG ? __ldcg(q) : __ldg(q);
+  const uint2 t = CG == kLdcg ? __ldcg(q) : __ldg(q);
+  const float2 a = __half22float2(*reinterpret_cast<const __half2 *>(&t.x));
+  const float2 b = __half22float2(*reinterpret_cast<const __half2 *>(&t.y));
+  return Quad<float>{{a.x, a.y, b.x, b.y}};
+}
+
+// The same from shared memory.
+__device__ __forceinline__ Quad<float> ldq_s(const float *p) {
+  const float4 t = *reinterpret_cast<const float4 *>(p);
+  return Quad<float>{{t.x, t.y, t.z, t.w}};
+}
+__device__ __forceinline__ Quad<float> ldq_s(const __nv_bfloat16 *p) {
+  const uint2 t = *reinterpret_cast<const uint2 *>(p);
+  return Quad<float>{{__uint_as_float(t.x << 16), __uint_as_float(t.x & 0xffff0000u),
+                      __uint_as_float(t.y << 16), __uint_as_float(t.y & 0xffff0000u)}};
+}
+__device__ __forceinline__ Quad<float> ldq_s(const __half *p) {
+  const uint2 t = *reinterpret_cast<const uint2 *>(p);
   const float2 a = __half22float2(*reinterpret_cast<const __half2 *>(&t.x));
   const float2 b = __half22float2(*reinterpret_cast<const __half2 *>(&t.y));
   return Quad<float>{{a.x, a.y, b.x, b.y}};
@@ -264,6 +292,8 @@ template <typename F> struct KArgsT {
   int wall_dir;             // bit 3 k + s: scalar s fixed to Cwall[k][s] on wall k
   F Cwall[3][3];            // k: 0 the x = 0 end, 1 the x = nx - 1 end, 2 the bottom
   int npal;                 // palette entries (the bounds-checked build tests indices)
+  int pair_rows;            // weighted rows of a unit's chunk in the two-step kernel
+  int pair_ahead;           // rows its warps prefetch into the L2 cache (0: none)
 };
 using KArgs = KArgsT<double>;
 
@@ -280,7 +310,7 @@ template <typename F> __host__ __device__ inline KArgsT<F> narrow_args(const KAr
   r.h_ch = F(a.h_ch); r.Q3 = F(a.Q3);
   r.inlet_pressure = a.inlet_pressure; r.dp_in = F(a.dp_in);
   r.gam_x = F(a.gam_x); r.gam_y = F(a.gam_y); r.buoy_off = F(a.buoy_off);
-  r.closed_x = a.closed_x; r.wall_dir = a.wall_dir; r.npal = a.npal;
+  r.closed_x = a.closed_x; r.wall_dir = a.wall_dir; r.npal = a.npal; r.pair_rows = a.pair_rows; r.pair_ahead = a.pair_ahead;
   r.halo_lo = a.halo_lo; r.halo_hi = a.halo_hi;
   for (int k = 0; k < 3; ++k)
     for (int s = 0; s < 3; ++s) r.Cwall[k][s] = F(a.Cwall[k][s]);
@@ -373,7 +403,7 @@ template <typename R> __device__ __forceinline__ R lam9(int i) {
 }
 
 // Population planes of one buffer; CG selects L2-only loads.
-template <typename S, bool CG = false> struct Pops {
+template <typename S, int CG = kLdg> struct Pops {
   const S *__restrict__ p;
   long long plane;
   int nxp;
@@ -384,6 +414,26 @@ template <typename S, bool CG = false> struct Pops {
     if (!in_bounds(i, pop_extent(plane, nxp), 1)) return V(0);
 #endif
     return ldp<CG>(p + pop_index(q, (long long)y * nxp + x, plane));
+  }
+};
+
+// The row ring that a warp of the two-step kernel (k_step2) keeps in shared
+// memory: the kRingRows newest rows of its kRingCols columns, laid out like a
+// population buffer (pop_index) whose planes are the ring.  Lattice row
+// y >= -1 is ring row (y + 1) mod kRingRows, lattice column x ring column
+// x - x_lo.  Plain loads (the warp writes the ring itself).
+constexpr int kRingRows = 3, kRingCols = 32, kRingCells = kRingRows * kRingCols;
+template <typename S> struct Pops<S, kRing> {
+  const S *p;
+  int x_lo;
+  static __device__ __forceinline__ int row(int y) { return (int)((unsigned)(y + 1) % kRingRows) * kRingCols; }
+  __device__ __forceinline__ auto at(int q, int x, int y) const {
+    const int c = row(y) + x - x_lo;
+#ifdef PEMLBM_BOUNDS_CHECK
+    using V = decltype(ld_s(p));
+    if (!in_bounds(x - x_lo, kRingCols, 5)) return V(0);
+#endif
+    return ld_s(p + (int)pop_index(q, c, kRingCells));
   }
 };
 
@@ -404,7 +454,7 @@ template <typename R> __device__ __forceinline__ R inlet_u(const KArgsT<R> &a, R
 // `v` is the interior pull already loaded for this link.  X: the extended
 // set-ups (closed x ends, fixed wall values, buoyancy) are compiled in; the
 // cathode's own step kernels are built without them.
-template <typename S, typename R, bool CG = false, bool X = false>
+template <typename S, typename R, int CG = kLdg, bool X = false>
 __device__ R pull_flow_edge(const Pops<S, CG> &src, const KArgsT<R> &a, const uint8_t *__restrict__ mask,
                             const uint16_t *__restrict__ mid, const MatCoef<R> *__restrict__ pal,
                             int i, int x, int y, uint8_t m, R v) {
@@ -469,7 +519,7 @@ __device__ __forceinline__ R wall_value(const KArgsT<R> &a, const MatCoef<R> &mc
 
 // Scalar link i of scalar s into cell (x, y); the bottom wall returns the
 // insulated (or, with X, fixed) value and the reaction is applied afterwards.
-template <typename S, typename R, bool CG = false, bool X = false>
+template <typename S, typename R, int CG = kLdg, bool X = false>
 __device__ R pull_scalar_edge(const Pops<S, CG> &src, const KArgsT<R> &a, const uint8_t *__restrict__ mask,
                               const MatCoef<R> &mc, int s, int i, int x, int y, uint8_t m, R v) {
   const int EX[5] = {0, 1, 0, -1, 0}, EY[5] = {0, 0, 1, 0, -1}, OP[5] = {0, 3, 4, 1, 2};
@@ -548,7 +598,7 @@ __device__ __forceinline__ R d2q5_sum(R d0, R d1, R d2, R d3, R d4) {
   return d0 + ((d1 + d3) + (d2 + d4));
 }
 
-template <typename S, typename R, bool CG = false>
+template <typename S, typename R, int CG = kLdg>
 __device__ __forceinline__ R own_sum(const Pops<S, CG> &src, int s, int x, int y) {
   const int q = 9 + 5 * s;
   return d2q5_sum<R>(R(src.at(q, x, y)), R(src.at(q + 1, x, y)), R(src.at(q + 2, x, y)),
@@ -558,7 +608,7 @@ __device__ __forceinline__ R own_sum(const Pops<S, CG> &src, int s, int x, int y
 // Surface reaction of the thin film at a bottom cell (Sec. 4): the implicit
 // Tafel link.  Returns the O2 consumed J (lattice units) and modifies the
 // three upward links.  theta_n = T^n - T_in from the cell's own state.
-template <typename S, typename R, bool CG = false>
+template <typename S, typename R, int CG = kLdg>
 __device__ __forceinline__ R surface_reaction(const Pops<S, CG> &src, const KArgsT<R> &a,
                                               const MatCoef<R> &mc, int x, Cell<R> &c) {
   R theta = own_sum<S, R, CG>(src, 0, x, 0) + a.theta0;
@@ -575,7 +625,7 @@ __device__ __forceinline__ R surface_reaction(const Pops<S, CG> &src, const KArg
 }
 
 // Volumetric catalyst sink of a catalyst cell (backward Euler in C).
-template <typename S, typename R, bool CG = false>
+template <typename S, typename R, int CG = kLdg>
 __device__ __forceinline__ R volume_sink(const Pops<S, CG> &src, const KArgsT<R> &a, int x, int y) {
   R theta = own_sum<S, R, CG>(src, 0, x, y) + a.theta0;
   R C = own_sum<S, R, CG>(src, 1, x, y) + R(a.Cref[1]);
@@ -585,7 +635,7 @@ __device__ __forceinline__ R volume_sink(const Pops<S, CG> &src, const KArgsT<R>
 }
 
 // The 24 interior pulls of cell (x, y), issued without looking at the mask.
-template <typename S, typename R, bool CG = false>
+template <typename S, typename R, int CG = kLdg>
 __device__ __forceinline__ void load_interior(const Pops<S, CG> &src, const KArgsT<R> &a, int x, int y,
                                               Cell<R> &c) {
   const long long c0 = (long long)y * a.nxp + x, P = a.plane, W = a.nxp;
@@ -623,8 +673,101 @@ __device__ __forceinline__ void load_interior(const Pops<S, CG> &src, const KArg
   c.f[8] = ldp<CG>(d + 3 * P + W - 1);
 }
 
+// The interior pulls of a cell, asked for well before they are used: the five
+// groups (and in FP32 the four diagonals) are copied asynchronously into the
+// lane's own slots of the warp's stage in shared memory, 16-bit diagonals
+// (too narrow for such a copy) wait in registers.  A lane reads back only
+// what it copied itself.
+template <typename S> struct Stage {
+  static constexpr int kGroup = 4 * (int)sizeof(S);                       // bytes of a group
+  static constexpr int kDiag = sizeof(S) == 4 ? 4 * 32 * (int)sizeof(S) : 0;
+  static constexpr int kBytes = 5 * 32 * kGroup + kDiag;                  // of one warp
+};
+template <int N> __device__ __forceinline__ void copy_async(void *smem, const void *g) {
+  const unsigned d = (unsigned)__cvta_generic_to_shared(smem);
+  if constexpr (N == 16) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(g) : "memory");
+  else asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(d), "l"(g), "n"(N) : "memory");
+}
+// c: the cell's index in the buffer
+template <typename S, typename R>
+__device__ __forceinline__ void request_interior(const Pops<S, kLdg> &src, const KArgsT<R> &a, unsigned c,
+                                                 int lane, unsigned char *stage, S (&diag)[4]) {
+  constexpr int G = Stage<S>::kGroup;
+  const long long P = a.plane, W = a.nxp;
+#ifdef PEMLBM_BOUNDS_CHECK
+  const long long n = pop_extent(P, a.nxp), k = c;
+  if (!in_bounds(4 * k, n, 2) || !in_bounds(4 * (P + k - 1), n, 2) || !in_bounds(4 * (2 * P + k - W), n, 2) ||
+      !in_bounds(4 * (4 * P + k + W) + 3, n, 2) || !in_bounds(20 * P + k - W - 1, n, 3) ||
+      !in_bounds(21 * P + k - W + 1, n, 3) || !in_bounds(22 * P + k + W + 1, n, 3) ||
+      !in_bounds(23 * P + k + W - 1, n, 3))
+    return;
+#endif
+  // one uniform base per plane and a 32-bit byte offset per lane
+  const char *p = reinterpret_cast<const char *>(src.p);
+  const unsigned og = c * (unsigned)G, od = c * (unsigned)sizeof(S);
+  auto group = [&](int i, long long from) {
+    copy_async<G>(stage + (i * 32 + lane) * G, p + (i * P + from) * G + og);
+  };
+  group(0, 0);
+  group(1, -1);
+  group(2, -W);
+  group(3, 1);
+  group(4, W);
+  const long long from[4] = {-W - 1, -W + 1, W + 1, W - 1};
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const char *q = p + ((20 + i) * P + from[i]) * (long long)sizeof(S) + od;
+    if constexpr (sizeof(S) == 4) copy_async<4>(stage + 5 * 32 * G + (i * 32 + lane) * 4, q);
+    else diag[i] = __ldg(reinterpret_cast<const S *>(q));
+  }
+  asm volatile("cp.async.commit_group;" ::: "memory");
+}
+template <typename S, typename R>
+__device__ __forceinline__ void take_interior(int lane, const unsigned char *stage, const S (&diag)[4],
+                                              Cell<R> &c) {
+  constexpr int G = Stage<S>::kGroup;
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
+#pragma unroll
+  for (int i = 0; i < 5; ++i) {
+    const auto v = ldq_s(reinterpret_cast<const S *>(stage + (i * 32 + lane) * G));
+    c.f[i] = v.v[0];
+    c.g[0][i] = v.v[1];
+    c.g[1][i] = v.v[2];
+    c.g[2][i] = v.v[3];
+  }
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    if constexpr (sizeof(S) == 4)
+      c.f[5 + i] = ld_s(reinterpret_cast<const S *>(stage + 5 * 32 * G + (i * 32 + lane) * 4));
+    else c.f[5 + i] = ld_s(&diag[i]);
+  }
+}
+
+// The same from the row ring, given the ring cells lo, c0, hi of the cell
+// below, the cell itself and the cell above.  (Ring column 0 and the last
+// have no neighbour on one side and are not pulled into.)
+template <typename S, typename R>
+__device__ __forceinline__ void load_interior(const Pops<S, kRing> &src, int lo, int c0, int hi,
+                                              Cell<R> &c) {
+  constexpr int P = kRingCells;
+  const int from[5] = {c0, c0 - 1, lo, c0 + 1, hi};
+#pragma unroll
+  for (int i = 0; i < 5; ++i) {
+    const auto v = ldq_s(src.p + 4 * (i * P + from[i]));
+    c.f[i] = v.v[0];
+    c.g[0][i] = v.v[1];
+    c.g[1][i] = v.v[2];
+    c.g[2][i] = v.v[3];
+  }
+  const S *d = src.p + 20 * P;
+  c.f[5] = ld_s(d + lo - 1);
+  c.f[6] = ld_s(d + P + lo + 1);
+  c.f[7] = ld_s(d + 2 * P + hi + 1);
+  c.f[8] = ld_s(d + 3 * P + hi - 1);
+}
+
 // The cell's own 24 stored values (no streaming), by groups.
-template <typename S, typename R, bool CG = false>
+template <typename S, typename R, int CG = kLdg>
 __device__ __forceinline__ void load_own(const Pops<S, CG> &src, int x, int y, Cell<R> &c) {
   const long long c0 = (long long)y * src.nxp + x, P = src.plane;
 #pragma unroll
@@ -654,10 +797,29 @@ __device__ __forceinline__ void load_own(const Pops<S, CG> &src, int x, int y, C
   }
 }
 
+// Cells whose only edge bit is M_NEAR_SOLID: a link whose source is a solid
+// grain takes the cell's own population of the opposite link (bounce-back,
+// as pull_flow_edge and pull_scalar_edge do); nb holds the solid sources
+// (bit i - 1 for link i of Eq. 2; the D2Q5 links are the first four).
+template <typename S, typename R, int CG = kLdg>
+__device__ __forceinline__ void bounce_solid(const Pops<S, CG> &src, int x, int y, uint32_t nb,
+                                             Cell<R> &c) {
+  const int OP[9] = OP9_TAB;
+#pragma unroll
+  for (int i = 1; i < 9; ++i)
+    if (nb & (1u << (i - 1))) c.f[i] = R(src.at(OP[i], x, y));
+#pragma unroll
+  for (int s = 0; s < 3; ++s)
+#pragma unroll
+    for (int i = 1; i < 5; ++i)
+      if (nb & (1u << (i - 1))) c.g[s][i] = R(src.at(9 + 5 * s + OP[i], x, y));
+}
+
 // Replaces the pulls of links that cross a wall, the inlet, the outlet, a
-// periodic seam or a solid grain (cells with any edge bit only).
-template <typename S, typename R, bool CG = false, bool X = false>
-__device__ __forceinline__ void fix_edges(const Pops<S, CG> &src, const KArgsT<R> &a,
+// periodic seam or a solid grain (cells with any edge bit only), link by
+// link: what a cell at the periodic seam needs.
+template <typename S, typename R, int CG = kLdg, bool X = false>
+__device__ __forceinline__ void fix_links(const Pops<S, CG> &src, const KArgsT<R> &a,
                                           const uint8_t *__restrict__ mask,
                                           const uint16_t *__restrict__ mid,
                                           const MatCoef<R> *__restrict__ pal,
@@ -673,26 +835,121 @@ __device__ __forceinline__ void fix_edges(const Pops<S, CG> &src, const KArgsT<R
       c.g[s][i] = pull_scalar_edge<S, R, CG, X>(src, a, mask, mc, s, i, x, y, m, c.g[s][i]);
 }
 
-// Cells whose only edge bit is M_NEAR_SOLID: a link whose source is a solid
-// grain takes the cell's own population of the opposite link (bounce-back,
-// as pull_flow_edge and pull_scalar_edge do); nb holds the solid sources
-// (bit i - 1 for link i of Eq. 2; the D2Q5 links are the first four).
-template <typename S, typename R, bool CG = false>
-__device__ __forceinline__ void bounce_solid(const Pops<S, CG> &src, int x, int y, uint32_t nb,
-                                             Cell<R> &c) {
-  const int OP[9] = OP9_TAB;
+// The value that flow link i takes from the virtual column -1 of the
+// pressure inlet or nx of the outlet at source row sy: the lattice's first or
+// last column vx with its equilibrium pressure part moved to phi p = 1/3
+// (+ dp), see pull_flow_edge.
+template <typename S, typename R, int CG>
+__device__ __forceinline__ R virtual_link(const Pops<S, CG> &src, const KArgsT<R> &a,
+                                          const uint16_t *__restrict__ mid,
+                                          const MatCoef<R> *__restrict__ pal, int i, int vx, int sy,
+                                          R dp) {
+  R d[9];
 #pragma unroll
-  for (int i = 1; i < 9; ++i)
-    if (nb & (1u << (i - 1))) c.f[i] = R(src.at(OP[i], x, y));
+  for (int k = 0; k < 9; ++k) d[k] = R(src.at(k, vx, sy));
+  R jx = d[1] - d[3] + d[5] - d[6] - d[7] + d[8];
+  R jy = d[2] - d[4] + d[5] + d[6] - d[7] - d[8];
+  R s18 = ((d[1] + d[3]) + (d[2] + d[4])) + ((d[5] + d[7]) + (d[6] + d[8]));
+  R inv_phi = pal[ld_mid(mid, (long long)sy * a.nxp + vx, a, 12)].inv_phi;
+  R dP = dp + (R(-0.6) * s18 + R(0.4) * (jx * jx + jy * jy) * inv_phi);
+  return d[i] + lam9<R>(i) * dP;
+}
+
+// The same as fix_links for a lattice that is not periodic, by node bits: a
+// side's code runs only where the cell lies on that side, and the links of
+// solid sources come from the second mask plane.  (Link by link, every edge
+// cell walks every branch of 20 links; the warps that own the lattice's end
+// columns then took several times an interior warp's time.)  Each link's
+// value is computed as there.
+template <typename S, typename R, int CG = kLdg, bool X = false>
+__device__ __forceinline__ void fix_edges(const Pops<S, CG> &src, const KArgsT<R> &a,
+                                          const uint8_t *__restrict__ mask,
+                                          const uint16_t *__restrict__ mid,
+                                          const MatCoef<R> *__restrict__ pal,
+                                          const MatCoef<R> &mc, int x, int y, uint8_t m,
+                                          Cell<R> &c) {
+  if constexpr (CG != kRing)
+    if (a.periodic) {
+      fix_links<S, R, CG, X>(src, a, mask, mid, pal, mc, x, y, m, c);
+      return;
+    }
+  // solid sources inside the lattice (also those in a neighbour slab)
+  if (m & M_NEAR_SOLID)
+    bounce_solid<S, R, CG>(src, x, y, ld_mask(mask, a.plane + (long long)y * a.nxp + x, a, 10), c);
+  if (m & M_XLO) {   // links 1, 5, 8; the D2Q5 link 1
+    const int in[3] = {1, 5, 8}, op[3] = {3, 7, 6}, ey[3] = {0, 1, -1};
+    const bool open = (m & M_INLET) != 0;
 #pragma unroll
-  for (int s = 0; s < 3; ++s)
+    for (int k = 0; k < 3; ++k) {
+      R w = R(src.at(op[k], x, y));
+      if (open && !a.inlet_pressure)
+        w += R(6) * w9<R>(in[k]) * R(1) * inlet_u<R>(a, R(y) - R(0.5) * R(ey[k]));
+      c.f[in[k]] = w;
+      if (open && a.inlet_pressure) {
+        const int sy = y - ey[k];
+        if (sy >= 0 && sy < a.ny && (ld_mask(mask, (long long)sy * a.nxp, a, 11) & M_INLET))
+          c.f[in[k]] = virtual_link<S, R, CG>(src, a, mid, pal, in[k], 0, sy, R(a.dp_in));
+      }
+    }
 #pragma unroll
-    for (int i = 1; i < 5; ++i)
-      if (nb & (1u << (i - 1))) c.g[s][i] = R(src.at(9 + 5 * s + OP[i], x, y));
+    for (int s = 0; s < 3; ++s) {
+      R w = R(src.at(9 + 5 * s + 3, x, y));
+      if (open) {
+        w = wall_value<R>(a, mc, s, w, R(a.Cin[s]));
+      } else if constexpr (X) {
+        if ((a.wall_dir >> s) & 1) w = wall_value<R>(a, mc, s, w, R(a.Cwall[0][s]));
+      }
+      c.g[s][1] = w;
+    }
+  }
+  if (m & M_XHI) {   // links 3, 6, 7; the D2Q5 link 3
+    const int in[3] = {3, 6, 7}, op[3] = {1, 8, 5}, ey[3] = {0, 1, -1};
+    const bool closed = X && a.closed_x;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const int sy = y - ey[k];
+      if (closed) c.f[in[k]] = R(src.at(op[k], x, y));
+      else if (sy >= 0 && sy < a.ny)
+        c.f[in[k]] = virtual_link<S, R, CG>(src, a, mid, pal, in[k], x, sy, R(0));
+    }
+#pragma unroll
+    for (int s = 0; s < 3; ++s) {
+      if (closed) {
+        R w = R(src.at(9 + 5 * s + 1, x, y));
+        if ((a.wall_dir >> (3 + s)) & 1) w = wall_value<R>(a, mc, s, w, R(a.Cwall[1][s]));
+        c.g[s][3] = w;
+      } else {
+        c.g[s][3] = R(src.at(9 + 5 * s + 3, x, y));   // fully developed
+      }
+    }
+  }
+  if (m & M_YLO) {   // links 2, 5, 6: the bottom wall
+    c.f[2] = R(src.at(4, x, y));
+    c.f[5] = R(src.at(7, x, y));
+    c.f[6] = R(src.at(8, x, y));
+#pragma unroll
+    for (int s = 0; s < 3; ++s) {
+      R w = R(src.at(9 + 5 * s + 4, x, y));
+      if constexpr (X)
+        if ((a.wall_dir >> (6 + s)) & 1) w = wall_value<R>(a, mc, s, w, R(a.Cwall[2][s]));
+      c.g[s][2] = w;
+    }
+  }
+  if (m & M_YHI) {   // links 4, 7, 8: the top wall
+    c.f[4] = R(src.at(2, x, y));
+    c.f[7] = R(src.at(5, x, y));
+    c.f[8] = R(src.at(6, x, y));
+#pragma unroll
+    for (int s = 0; s < 3; ++s) {
+      R w = R(src.at(9 + 5 * s + 2, x, y));
+      if (a.top_dirichlet) w = wall_value<R>(a, mc, s, w, R(a.Ctop[s]));
+      c.g[s][4] = w;
+    }
+  }
 }
 
 // Pull all 24 populations of a non-solid cell (x, y).
-template <typename S, typename R, bool CG = false, bool X = false>
+template <typename S, typename R, int CG = kLdg, bool X = false>
 __device__ __forceinline__ void pull_cell(const Pops<S, CG> &src, const KArgsT<R> &a,
                                           const uint8_t *__restrict__ mask,
                                           const uint16_t *__restrict__ mid,

@@ -34,7 +34,7 @@ __device__ __forceinline__ void stage_args(const BatchCaseT<R> *__restrict__ cas
     dstw[k] = __ldg(srcw + k);
 }
 
-template <typename S, int BX, int BY, bool CG>
+template <typename S, int BX, int BY, int CG>
 __device__ __forceinline__ void batch_tile(const BatchCaseT<typename Real<S>::type> *__restrict__ cases,
                                            const int *__restrict__ tile_start, int ncases, int t,
                                            int parity, KArgsT<typename Real<S>::type> *sa,
@@ -67,7 +67,28 @@ k_batch_step(const BatchCaseT<typename Real<S>::type> *__restrict__ cases,
              const int *__restrict__ tile_start, int ncases, int parity) {
   __shared__ KArgsT<typename Real<S>::type> sa;
   __shared__ int sc;
-  batch_tile<S, BX, BY, false>(cases, tile_start, ncases, blockIdx.x, parity, &sa, &sc);
+  batch_tile<S, BX, BY, kLdg>(cases, tile_start, ncases, blockIdx.x, parity, &sa, &sc);
+}
+
+// Two steps per launch (k_step2); block_start numbers the blocks of
+// kPairWarps strip x row chunk units case after case.
+template <typename S>
+__global__ void __launch_bounds__(32 * kPairWarps, pair_blocks_per_sm(sizeof(S)))
+k_batch_step2(const BatchCaseT<typename Real<S>::type> *__restrict__ cases,
+              const int *__restrict__ block_start, int ncases, int parity) {
+  using R = typename Real<S>::type;
+  __shared__ KArgsT<R> sa;
+  __shared__ int sc;
+  if (threadIdx.x == 0) sc = batch_case_of(block_start, ncases, blockIdx.x);
+  __syncthreads();
+  const int c = sc;
+  stage_args(cases, c, &sa);
+  __syncthreads();
+  const BatchCaseT<R> &bc = cases[c];
+  const int cur = bc.cur0 ^ parity;
+  two_steps_unit<S, false, false>(
+      (const S *)bc.pop[cur], (S *)bc.pop[cur ^ 1], bc.mask, bc.mid, (const MatCoef<R> *)bc.pal, sa,
+      (blockIdx.x - __ldg(block_start + c)) * kPairWarps + (threadIdx.x >> 5), (R *)nullptr, 0);
 }
 
 // Grid-wide barrier of a cooperative launch.  Every wait is bounded: after
@@ -112,7 +133,7 @@ k_batch_persistent(const BatchCaseT<typename Real<S>::type> *__restrict__ cases,
   __shared__ int sc;
   for (int step = 0; step < nsteps; ++step) {
     for (int t = blockIdx.x; t < total_tiles; t += gridDim.x)
-      batch_tile<S, BX, BY, true>(cases, tile_start, ncases, t, step & 1, &sa, &sc);
+      batch_tile<S, BX, BY, kLdcg>(cases, tile_start, ncases, t, step & 1, &sa, &sc);
     if (!grid_barrier(bar, bar + 1, gridDim.x, status, spin_limit)) return;
   }
 }
@@ -137,7 +158,7 @@ __global__ void k_fields(const S *__restrict__ src_p, const uint8_t *__restrict_
   const Pops<S> src{src_p, a.plane, a.nxp};
   const MatCoef<R> mc = pal[mid[c]];
   Cell<R> cell;
-  pull_cell<S, R, false, true>(src, a, mask, mid, pal, mc, x, y, m, cell);
+  pull_cell<S, R, kLdg, true>(src, a, mask, mid, pal, mc, x, y, m, cell);
   if (a.mode == 0 && (m & M_YLO)) surface_reaction<S, R>(src, a, mc, x, cell);
   const Macro<R> u = macros<R, true>(a, mc, cell);
   out[0 * n + o] = (double)u.ux;
@@ -205,7 +226,7 @@ k_balances(const S *__restrict__ src_p, const uint8_t *__restrict__ mask,
           const int sy = y - EY[i];
           if (EX[i] == dir) {                       // enters through the column
             if (sy < 0 || sy >= a.ny) continue;     // a wall link
-            const R v = pull_flow_edge<S, R, false, true>(src, a, mask, mid, pal, i, x, y, m, R(0));
+            const R v = pull_flow_edge<S, R, kLdg, true>(src, a, mask, mid, pal, i, x, y, m, R(0));
             // inlet: the pulled value replaces the bounced one (the moving-wall
             // or virtual-column excess); outlet: the whole pulled value
             o[0] += side ? (double)v : (double)v - (double)R(src.at(OP[i], x, y));
@@ -218,7 +239,7 @@ k_balances(const S *__restrict__ src_p, const uint8_t *__restrict__ mask,
         for (int s = 0; s < 3; ++s) {
           const int q = 9 + 5 * s;
           const int lin = side ? 3 : 1;              // D2Q5 link entering through the column
-          const R v = pull_scalar_edge<S, R, false, true>(src, a, mask, mc, s, lin, x, y, m, R(0));
+          const R v = pull_scalar_edge<S, R, kLdg, true>(src, a, mask, mc, s, lin, x, y, m, R(0));
           if (side) {
             o[1 + s] += (double)v - (double)R(src.at(q + 1, x, y));   // in via 3, out via 1
           } else if ((m & M_INLET) || ((a.wall_dir >> s) & 1)) {
@@ -290,7 +311,34 @@ k_catalyst(const S *__restrict__ src_p, const uint8_t *__restrict__ mask,
   }
 }
 
-// Sums the per-column J and heat in a fixed order: out[0], out[1].
+// The same sums of observed steps from the reaction each step wrote itself:
+// jcells [step][rows][nx] holds the O2 a cell consumed in a step (0 for cells
+// that do not react), rows in the order and grouping of k_catalyst.  One row
+// of blocks per step; colsum [step][2][nx].
+template <typename R>
+__global__ void __launch_bounds__(kCatalystBX * kCatalystBY)
+k_sum_cells(const R *__restrict__ jcells, int nx, int rows, double hpo, double *__restrict__ colsum) {
+  __shared__ double sm[kCatalystBY][kCatalystBX];
+  const int tx = threadIdx.x % kCatalystBX, ty = threadIdx.x / kCatalystBX;
+  const int x = blockIdx.x * kCatalystBX + tx;
+  const R *j = jcells + (long long)blockIdx.y * rows * nx;
+  double J = 0.0;
+  if (x < nx)
+#pragma unroll 4
+    for (int y = ty; y < rows; y += kCatalystBY) J += (double)j[(long long)y * nx + x];
+  sm[ty][tx] = J;
+  __syncthreads();
+  if (ty == 0 && x < nx) {
+    double t = 0.0;
+    for (int k = 0; k < kCatalystBY; ++k) t += sm[k][tx];
+    double *c = colsum + (long long)blockIdx.y * 2 * nx;
+    c[x] = t;
+    c[nx + x] = t * (double)(R)hpo;
+  }
+}
+
+// Sums the per-column J and heat in a fixed order: out[0], out[1]; block k
+// those of step k.
 __global__ void k_sum_columns(const double *__restrict__ colsum, int nx, double *__restrict__ out);
 
 // ------------------------------------------------- residual (K4)
@@ -463,6 +511,29 @@ void launch_batch_step(const BatchCase *cases, const int *tile_start, int ncases
   }
 }
 
+template <typename S>
+void launch_batch_step2(const BatchCase *cases, const int *block_start, int ncases, int blocks,
+                        int parity, cudaStream_t st) {
+  if constexpr (sizeof(S) < 8)
+    k_batch_step2<S><<<blocks, 32 * kPairWarps, pair_smem_bytes(sizeof(S)), st>>>(
+        (const BatchCaseT<typename Real<S>::type> *)cases, block_start, ncases, parity);
+}
+
+// Opts the two-step kernels into their shared memory on the current device.
+template <typename S>
+cudaError_t allow_step2() {
+  if constexpr (sizeof(S) < 8) {
+    const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
+    const int n = (int)pair_smem_bytes(sizeof(S));
+    cudaError_t e = cudaFuncSetAttribute(k_step2<S, false, false>, attr, n);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_step2<S, false, true>, attr, n);
+    if constexpr (sizeof(S) == 2)
+      if (e == cudaSuccess) e = cudaFuncSetAttribute(k_step2<S, true, false>, attr, n);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_batch_step2<S>, attr, n);
+    return e;
+  }
+  return cudaSuccess;
+}
 
 template <typename S>
 cudaError_t launch_batch_persistent(const BatchCase *cases, const int *tile_start, int ncases,
@@ -640,7 +711,10 @@ template <typename S> unsigned long long bounds_first_bad() {
 #define PEMLBM_INSTANTIATE(S)                                                                   \
   template unsigned long long bounds_first_bad<S>();                                           \
   template void launch_step<S>(const void *, void *, const DevGeom &, const KArgs &, int,       \
-                               cudaStream_t);                                                   \
+                               void *, cudaStream_t);                                           \
+  template void launch_step2<S>(const void *, void *, const DevGeom &, const KArgs &, void *,    \
+                                long long, cudaStream_t);                                       \
+  template cudaError_t allow_step2<S>();                                                   \
   template void launch_fields<S>(const void *, const DevGeom &, const KArgs &, double *,        \
                                  cudaStream_t);                                                 \
   template void launch_balances<S>(const void *, const DevGeom &, const KArgs &, double *,      \
@@ -656,6 +730,8 @@ template <typename S> unsigned long long bounds_first_bad() {
                                     cudaStream_t);                                              \
   template void launch_batch_step<S>(const BatchCase *, const int *, int, int, int, int,        \
                                      cudaStream_t);                                             \
+  template void launch_batch_step2<S>(const BatchCase *, const int *, int, int, int,            \
+                                      cudaStream_t);                                            \
   template cudaError_t launch_batch_persistent<S>(const BatchCase *, const int *, int, int, int, \
                                                   unsigned *, int *, long long, cudaStream_t);  \
   template void batch_upload<S>(const BatchCase *, int, void *, void *, cudaStream_t);         \

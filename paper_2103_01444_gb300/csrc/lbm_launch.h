@@ -19,6 +19,23 @@ constexpr int kStepVariants = 8;
 constexpr StepShape kStepShapes[kStepVariants] = {
     {128, 2, 1}, {128, 2, 3}, {128, 2, 4}, {64, 4, 4},
     {256, 1, 4}, {32, 8, 4}, {128, 1, 8}, {64, 2, 8}};
+// Shape of the two-step kernel: a warp per strip of kStripCols columns (its
+// first step covers one column more on either side) and chunk of rows.  Its
+// shared memory holds a ring of three rows of 24 populations per lane and
+// the stage of the row on its way (Stage).  FP32: 16 warps per SM at 122
+// registers (limited by shared memory); 16 bits: 20 warps at 96.  With more
+// warps the kernel spills, and beside the rings there is little L1 cache left
+// to hold what it spills (4096 x 1024, us a step: FP32 16 / 18 warps 81 / 88,
+// BF16 20 / 24 warps 74 / 80).
+constexpr int kStripCols = 30, kPairWarps = 2;
+constexpr size_t pair_smem_bytes(size_t esize) {
+  return (size_t)kPairWarps * (96 * 24 * esize + 32 * (esize == 4 ? 24 : 20) * esize);
+}
+constexpr int pair_blocks_per_sm(size_t esize) { return esize == 4 ? 8 : 10; }
+// Weighted rows of a unit's chunk for one lattice or the cases of a batch, and
+// a lattice's blocks.
+int pair_rows(const int *nx, const int *ny, const int *ny_cl, int n, size_t esize);
+int pair_blocks(int nx, int ny, int ny_cl, int rows);
 constexpr int kReduceThreads = 512;
 // Persistent batched step: 128 x 1 cells per block, 8 blocks per SM asked of
 // the register allocator; the grid is the number of co-resident blocks.
@@ -41,7 +58,9 @@ struct DevGeom {
   const void *pal;       // MatCoef<R>[npal]
 };
 
-template <typename S> void launch_step(const void *src, void *dst, const DevGeom &g, const KArgs &a, int variant, cudaStream_t st);
+template <typename S> void launch_step(const void *src, void *dst, const DevGeom &g, const KArgs &a, int variant, void *jout, cudaStream_t st);
+template <typename S> cudaError_t allow_step2();
+template <typename S> void launch_step2(const void *src, void *dst, const DevGeom &g, const KArgs &a, void *jout, long long jstep, cudaStream_t st);
 // Reverse records of one step (device pointers, the arithmetic type of the
 // domain; layout as RecPtrs in lbm_core.cuh).
 struct RecBufs {
@@ -53,6 +72,9 @@ template <typename S> void launch_step_rec(const void *src, void *dst, const Dev
 template <typename S> void launch_fields(const void *src, const DevGeom &g, const KArgs &a, double *out, cudaStream_t st);
 template <typename S> void launch_balances(const void *src, const DevGeom &g, const KArgs &a, double *out, cudaStream_t st);
 template <typename S> void launch_catalyst(const void *src, const DevGeom &g, const KArgs &a, double i_scale, float *profile, double *colsum, double *out, cudaStream_t st);
+// (J, heat) of nsteps observed steps from what their cells consumed
+// ([step][rows][nx], arithmetic precision) into out [step][2].
+void launch_sum_reaction(const void *jcells, bool fp64, int nx, int rows, int nsteps, double hpo, double *colsum, double *out, cudaStream_t st);
 // Residual of state src against snap_in, writing the new snapshot to snap_out
 // (the same buffer for an in-place update).
 template <typename S> void launch_residual(const void *src, const DevGeom &g, const KArgs &a, const void *snap_in, void *snap_out, double *partial, int *bad, double *out, cudaStream_t st);
@@ -66,6 +88,7 @@ template <typename S> void launch_set_state(void *pop, const DevGeom &g, const K
 
 template <typename S> void batch_upload(const BatchCase *host, int n, void *staging, void *dev, cudaStream_t st);
 template <typename S> void launch_batch_step(const BatchCase *cases, const int *tile_start, int ncases, int total_tiles, int variant, int parity, cudaStream_t st);
+template <typename S> void launch_batch_step2(const BatchCase *cases, const int *block_start, int ncases, int blocks, int parity, cudaStream_t st);
 template <typename S> cudaError_t launch_batch_persistent(const BatchCase *cases, const int *tile_start, int ncases, int total_tiles, int nsteps, unsigned *bar, int *status, long long spin_limit, cudaStream_t st);
 
 // Buffers of one reverse step (types follow the domain's arithmetic).
@@ -91,8 +114,8 @@ template <typename S> void launch_adj_seed_current(const void *src, const DevGeo
 // the plain build), cleared when read.
 template <typename S> unsigned long long bounds_first_bad();
 
-// Advances the step counter that seeds stochastic 16-bit rounding.
-void launch_seed_advance(unsigned *ctr, cudaStream_t st);
+// Advances by n the step counter that seeds stochastic 16-bit rounding.
+void launch_seed_advance(unsigned *ctr, unsigned n, cudaStream_t st);
 
 // Material palette built on the device from per-cell fields in device
 // memory ([ny][nx] doubles; sigma may be NULL = 1): the distinct tuples in

@@ -3,6 +3,8 @@
 // the read-out, batch and adjoint kernels so that its sources can be
 // identified on their own.
 #pragma once
+#include <type_traits>
+
 #include "lbm_core.cuh"
 #include "lbm_launch.h"
 
@@ -11,7 +13,7 @@ namespace pemlbm {
 // Own-state and pulled records of a listed cell (see RecPtrs): the values
 // the reverse of its reaction and of its boundary links needs.  `cell`
 // holds the post-stream values before the surface reaction.
-template <typename S, typename R, bool CG>
+template <typename S, typename R, int CG>
 __device__ __forceinline__ void write_listed_records(const Pops<S, CG> &src, const KArgsT<R> &a,
                                                      const RecPtrs<R> &rp, uint8_t m, long long c,
                                                      int x, int y, const Cell<R> &cell) {
@@ -41,39 +43,61 @@ __device__ __forceinline__ void write_listed_records(const Pops<S, CG> &src, con
 }
 
 // ------------------------------------------------------------- step (K1)
-// One coupled update of cell (x, y): src -> dst.  Shared by the single-
-// domain step and the batched steps.  X: closed ends, fixed wall values and
-// buoyancy compiled in (see pull_flow_edge).  REC: the step also writes
-// its reverse records (RecPtrs) for the discrete adjoint.
-template <typename S, bool CG = false, bool SR = false, bool X = false, bool REC = false>
-__device__ __forceinline__ void cell_update(const S *__restrict__ src_p, S *__restrict__ dst,
+// The update of cell (x, y) once its interior pulls are in `cell`: boundary
+// links, reaction, collisions, store.  c is its index in the lattice, m its
+// node bits; the 24 new values go to cell k of dst, a buffer whose planes
+// hold P cells (I = unsigned: the lattice's planes, addressed by one uniform
+// base per plane and a 32-bit byte offset).  jout, when not NULL, is where
+// reacting cells leave the O2 they consume in this step, [row][nx]; write_j
+// says whether this cell's caller owns it.  seed: the step counter of
+// stochastic rounding.
+// Shared by the single-domain step, the batched steps and the two-step
+// kernel.  X: closed ends, fixed wall values and buoyancy compiled in (see
+// pull_flow_edge).  REC: the step also writes its reverse records
+// (RecPtrs) for the discrete adjoint.
+template <typename S, int CG, bool SR, bool X, bool REC, typename I>
+__device__ __forceinline__ void finish_cell(const Pops<S, CG> &src, S *__restrict__ dst, I k, I P,
                                             const uint8_t *__restrict__ mask,
                                             const uint16_t *__restrict__ mid,
                                             const MatCoef<typename Real<S>::type> *__restrict__ pal,
-                                            const KArgsT<typename Real<S>::type> &a, int x,
-                                            int y,
-                                            const RecPtrs<typename Real<S>::type> &rp = {}) {
+                                            const KArgsT<typename Real<S>::type> &a, long long c,
+                                            int x, int y, uint8_t m,
+                                            const MatCoef<typename Real<S>::type> &mc,
+                                            Cell<typename Real<S>::type> &cell,
+                                            typename Real<S>::type *__restrict__ jout,
+                                            bool write_j, unsigned seed,
+                                            const RecPtrs<typename Real<S>::type> &rp) {
   using R = typename Real<S>::type;
-  const long long c = (long long)y * a.nxp + x;
-  const Pops<S, CG> src{src_p, a.plane, a.nxp};
-  const uint8_t m = ld_mask(mask, c, a, 20);
-  Cell<R> cell;
-  load_interior<S, R, CG>(src, a, x, y, cell);
   // solid cells run the same arithmetic on their (unused) values and only
   // skip the stores, so no branch stands between the mask and the loads
   const bool live = (m & REG_MASK) != REG_SOLID;
-  const MatCoef<R> mc = pal[ld_mid(mid, c, a, 21)];
-  if (m & M_EDGE) {
+  auto edges = [&] {
     // next to grains but away from the lattice's edges: bounce-back only
     if ((m & M_EDGE) == M_NEAR_SOLID)
       bounce_solid<S, R, CG>(src, x, y, ld_mask(mask, a.plane + c, a, 23), cell);
     else fix_edges<S, R, CG, X>(src, a, mask, mid, pal, mc, x, y, m, cell);
-  }
-  if constexpr (REC)
-    if (live) write_listed_records<S, R, CG>(src, a, rp, m, c, x, y, cell);
-  if (a.mode == 0 && (m & M_YLO)) surface_reaction<S, R, CG>(src, a, mc, x, cell);
+  };
   R S_vol = 0;
-  if (a.mode == 1 && (m & REG_MASK) == REG_CATALYST) S_vol = volume_sink<S, R, CG>(src, a, x, y);
+  auto reaction = [&] {
+    if (a.mode == 0 && (m & M_YLO)) {
+      const R J = surface_reaction<S, R, CG>(src, a, mc, x, cell);
+      if (jout && write_j && live) jout[(long long)y * a.nx + x] = J;
+    }
+    if (a.mode == 1 && (m & REG_MASK) == REG_CATALYST) {
+      S_vol = volume_sink<S, R, CG>(src, a, x, y);
+      if (jout && write_j) jout[(long long)y * a.nx + x] = -S_vol;
+    }
+  };
+  if constexpr (REC) {
+    if (m & M_EDGE) edges();
+    if (live) write_listed_records<S, R, CG>(src, a, rp, m, c, x, y, cell);
+    reaction();
+  } else if ((m & M_EDGE) || (m & REG_MASK) == REG_CATALYST) {
+    // one branch for everything an interior cell of a layer without reaction
+    // skips (a surface reaction is on the bottom edge)
+    if (m & M_EDGE) edges();
+    reaction();
+  }
   const Macro<R> u = macros<R, X>(a, mc, cell);
   if constexpr (REC) {
     if (live) {
@@ -95,23 +119,36 @@ __device__ __forceinline__ void cell_update(const S *__restrict__ src_p, S *__re
   // against 2% with this assignment).
   unsigned rnd[12] = {};
   if constexpr (SR) {
-    unsigned rs = hash32((unsigned)c * 0x9e3779b9u ^ hash32(__ldg(a.seed_ctr) + 0x632be5abu)) | 1u;
+    unsigned rs = hash32((unsigned)c * 0x9e3779b9u ^ hash32(seed + 0x632be5abu)) | 1u;
 #pragma unroll
     for (int j = 0; j < 12; ++j) rnd[j] = xorshift32(rs);
   }
   auto r16 = [&](int q) { return (q & 1) ? rnd[q >> 1] >> 16 : rnd[q >> 1] & 0xffffu; };
-  const long long P = a.plane;
   // (the bounds-checked build skips a store outside the 24 planes)
-  auto st_ok = [&](long long k, int width) { return in_bounds(k, 24 * P, 24) && in_bounds(k + width - 1, 24 * P, 24); };
+  auto st_ok = [&](long long i, int width) {
+    const long long n = 24 * (long long)(std::is_same<I, unsigned>::value ? a.plane : P);
+    return in_bounds(i, n, 24) && in_bounds(i + width - 1, n, 24);
+  };
+  // where population q (a group's first, or a diagonal link) of cell k goes
+  auto at = [&](int q) {
+    if constexpr (std::is_same<I, unsigned>::value) {
+      const int n = q < 5 ? 4 : 1;
+      return reinterpret_cast<S *>(reinterpret_cast<char *>(dst) +
+                                   (q < 5 ? 4 * q : 15 + q) * a.plane * (long long)sizeof(S) +
+                                   k * (unsigned)(n * sizeof(S)));
+    } else {
+      return dst + (I)pop_index(q, k, P);
+    }
+  };
   if (live) {   // the diagonal flow links
     if constexpr (SR) {
 #pragma unroll
       for (int i = 5; i < 9; ++i)
-        if (st_ok(pop_index(i, c, P), 1)) st_sr(dst + pop_index(i, c, P), o[i], r16(i));
+        if (st_ok(pop_index(i, k, std::is_same<I, unsigned>::value ? a.plane : (long long)P), 1)) st_sr(at(i), o[i], r16(i));
     } else {
 #pragma unroll
       for (int i = 5; i < 9; ++i)
-        if (st_ok(pop_index(i, c, P), 1)) st_r(dst + pop_index(i, c, P), o[i]);
+        if (st_ok(pop_index(i, k, std::is_same<I, unsigned>::value ? a.plane : (long long)P), 1)) st_r(at(i), o[i]);
     }
   }
   const R srcv[3] = {-S_vol * R(a.hpo) * mc.inv_sigma, S_vol, R(-2) * S_vol};
@@ -122,15 +159,37 @@ __device__ __forceinline__ void cell_update(const S *__restrict__ src_p, S *__re
   if (live) {   // links 0-4 of the flow and the three scalars, one group each
 #pragma unroll
     for (int i = 0; i < 5; ++i) {
-      if (!st_ok(pop_index(i, c, P), 4)) continue;
+      if (!st_ok(pop_index(i, k, std::is_same<I, unsigned>::value ? a.plane : (long long)P), 4)) continue;
       if constexpr (SR) {
-        stq_sr(dst + pop_index(i, c, P), o[i], g[0][i], g[1][i], g[2][i], r16(i), r16(9 + i),
+        stq_sr(at(i), o[i], g[0][i], g[1][i], g[2][i], r16(i), r16(9 + i),
                r16(14 + i), r16(19 + i));
       } else {
-        stq(dst + pop_index(i, c, P), o[i], g[0][i], g[1][i], g[2][i]);
+        stq(at(i), o[i], g[0][i], g[1][i], g[2][i]);
       }
     }
   }
+}
+
+// One coupled update of cell (x, y) of a global buffer: src -> dst.
+template <typename S, int CG = kLdg, bool SR = false, bool X = false, bool REC = false>
+__device__ __forceinline__ void cell_update(const S *__restrict__ src_p, S *__restrict__ dst,
+                                            const uint8_t *__restrict__ mask,
+                                            const uint16_t *__restrict__ mid,
+                                            const MatCoef<typename Real<S>::type> *__restrict__ pal,
+                                            const KArgsT<typename Real<S>::type> &a, int x, int y,
+                                            typename Real<S>::type *__restrict__ jout = nullptr,
+                                            const RecPtrs<typename Real<S>::type> &rp = {}) {
+  using R = typename Real<S>::type;
+  const long long c = (long long)y * a.nxp + x;
+  const Pops<S, CG> src{src_p, a.plane, a.nxp};
+  const uint8_t m = ld_mask(mask, c, a, 20);
+  Cell<R> cell;
+  load_interior<S, R, CG>(src, a, x, y, cell);
+  const MatCoef<R> mc = pal[ld_mid(mid, c, a, 21)];
+  unsigned seed = 0;
+  if constexpr (SR) seed = __ldg(a.seed_ctr);
+  finish_cell<S, CG, SR, X, REC, long long>(src, dst, c, a.plane, mask, mid, pal, a, c, x, y, m, mc,
+                                            cell, jout, true, seed, rp);
 }
 
 // SR: 16-bit stores with stochastic rounding (a separate instantiation, so
@@ -139,11 +198,175 @@ template <typename S, int BX, int BY, int MINB, bool SR = false, bool X = false>
 __global__ void __launch_bounds__(BX * BY, MINB)
 k_step(const S *__restrict__ src_p, S *__restrict__ dst, const uint8_t *__restrict__ mask,
        const uint16_t *__restrict__ mid, const MatCoef<typename Real<S>::type> *__restrict__ pal,
-       KArgsT<typename Real<S>::type> a) {
+       KArgsT<typename Real<S>::type> a, typename Real<S>::type *__restrict__ jout) {
   const int x = blockIdx.x * BX + (threadIdx.x % BX);
   const int y = blockIdx.y * BY + (threadIdx.x / BX);
   if (x >= a.nx || y >= a.ny) return;
-  cell_update<S, false, SR, X>(src_p, dst, mask, mid, pal, a, x, y);
+  cell_update<S, kLdg, SR, X>(src_p, dst, mask, mid, pal, a, x, y, jout);
+}
+
+// -------------------------------------------------------- two steps (K1b)
+// Two coupled steps in one pass over memory: src -> (row ring) -> dst.  A
+// warp owns a strip of kStripCols columns and walks up the rows [ya, yb): a
+// round takes the first step of one row, of kRingCols columns (one more on
+// either side), into the ring, and the second step of the row below from
+// the ring to dst.  The two steps of a cell are exactly two single steps.
+//
+// A single step of this lattice is bound by HBM (FP32, 0.95 of the measured
+// copy rate at 4096 x 1024) or by latency and issue (16 bits); a pair moves
+// the same bytes for two steps and is bound by issue and by what is left of
+// the memory latency (FP32: 62% of issue slots, 2.0 of 5.6 warp cycles per
+// issue wait for loads).  One warp alone owns its ring, so no block barrier
+// ties warps in different phases together (with blocks of 128 x 2 cells and
+// __syncthreads: 184 us a step).  The next row's pulls are copied into the
+// stage while both steps of this round run, and a column's material stays in
+// registers.  Per step, two at a time against single steps (tuned shape in
+// 16 bits): 4096 x 1024 FP32 81.3 against 124.5 us, BF16 74.3 against 87;
+// 1024 x 256 FP32 9.7 against 11.5; 200 x 40 FP32 3.6 against 6.8.
+template <typename S, bool SR, bool X>
+__device__ __forceinline__ void two_steps(const S *__restrict__ src_p, S *__restrict__ dst,
+                                          const uint8_t *__restrict__ mask,
+                                          const uint16_t *__restrict__ mid,
+                                          const MatCoef<typename Real<S>::type> *__restrict__ pal,
+                                          const KArgsT<typename Real<S>::type> &a, int strip,
+                                          int ya, int yb, typename Real<S>::type *__restrict__ jout,
+                                          long long jstep, S *__restrict__ ring,
+                                          unsigned char *__restrict__ stage) {
+  using R = typename Real<S>::type;
+  const int lane = threadIdx.x & 31;
+  const int x0 = strip * kStripCols - 1, x = x0 + lane;
+  const bool in_x = x >= 0 && x < a.nx;
+  const bool own_x = in_x && lane >= 1 && lane <= kStripCols;
+  const Pops<S, kLdg> src{src_p, a.plane, a.nxp};
+  const Pops<S, kRing> between{ring, x0};
+  unsigned seed = 0;
+  if constexpr (SR) seed = __ldg(a.seed_ctr);
+  R *const jout2 = jout ? jout + jstep : nullptr;
+  const int y_top = yb < a.ny ? yb : a.ny - 1;   // the last row the second step pulls from
+  // this lane's cell in ring row y1 (row y1 - 1 follows two ring rows on,
+  // row y1 - 2 one), and its node bits and palette index in the rows y1 - 1
+  // and y1
+  int hi = between.row(ya - 1) + lane;
+  unsigned m_lo = REG_SOLID, m_hi = REG_SOLID, e_lo = 0, e_hi = 0;
+  unsigned c1 = (unsigned)(ya - 1) * (unsigned)a.nxp + (unsigned)x;   // cell (x, y1)
+  // the lines of a coming row that this lane prefetches into the L2 cache:
+  // five 128-byte lines of each group plane, one of each diagonal, palette
+  // indices and node bits
+  const long long pf_cell = (long long)(ya - 1 + a.pair_ahead) * a.nxp + (x0 > 0 ? x0 : 0);
+  const char *pf;
+  int pf_row;
+  if (lane < 25) {
+    pf = (const char *)(src_p + 4 * ((lane / 5) * a.plane + pf_cell)) + 128 * (lane % 5);
+    pf_row = a.nxp * 4 * (int)sizeof(S);
+  } else if (lane < 29) {
+    pf = (const char *)(src_p + (lane - 5) * a.plane + pf_cell);
+    pf_row = a.nxp * (int)sizeof(S);
+  } else if (lane == 29) {
+    pf = (const char *)(mid + pf_cell);
+    pf_row = 2 * a.nxp;
+  } else {
+    pf = (const char *)(mask + pf_cell);
+    pf_row = a.nxp;
+  }
+  const int pf_top = a.pair_ahead ? y_top - a.pair_ahead : -2;   // last row y1 that prefetches
+  S diag[4] = {};
+  if (in_x) {
+    const unsigned c = ya > 0 ? c1 : c1 + a.nxp;   // the first row taken
+    request_interior(src, a, c, lane, stage, diag);
+    m_hi = ld_mask(mask, c, a, 20);
+    e_hi = ld_mid(mid, c, a, 21);
+  }
+  // the material of a column changes rarely from row to row: its
+  // coefficients stay in registers until the palette index differs
+  MatCoef<R> mc{};
+  unsigned e_mc = ~0u;
+  auto material = [&](unsigned e) {
+    if (e != e_mc) {
+      mc = pal[e];
+      e_mc = e;
+    }
+  };
+  for (int y1 = ya - 1; y1 <= yb; ++y1, c1 += a.nxp) {
+    unsigned m_next = REG_SOLID, e_next = 0;
+    if (y1 <= pf_top) asm volatile("prefetch.global.L2 [%0];" ::"l"(pf));
+    pf += pf_row;
+    const bool first = in_x && y1 >= 0 && y1 <= y_top;
+    if (first) {   // first step of row y1
+      Cell<R> cell;
+      take_interior<S, R>(lane, stage, diag, cell);
+      material(e_hi);
+      // the next row is on its way during both steps (past the last row, the
+      // last one again: nothing takes it)
+      const unsigned c2 = c1 + (y1 < y_top ? a.nxp : 0);
+      request_interior(src, a, c2, lane, stage, diag);
+      m_next = ld_mask(mask, c2, a, 20);
+      e_next = ld_mid(mid, c2, a, 21);
+      finish_cell<S, kLdg, SR, X, false, int>(
+          src, ring, hi, kRingCells, mask, mid, pal, a, c1, x, y1, (uint8_t)m_hi, mc, cell, jout,
+          own_x && y1 >= ya && y1 < yb, seed, RecPtrs<R>{});
+    }
+    __syncwarp();
+    const int y = y1 - 1;
+    if (own_x && y >= ya) {   // second step of row y (y < yb)
+      const unsigned c = c1 - a.nxp;
+      const int lo = hi >= 2 * kRingCols ? hi - 2 * kRingCols : hi + kRingCols;
+      const int c0 = hi >= kRingCols ? hi - kRingCols : hi + 2 * kRingCols;
+      Cell<R> cell;
+      load_interior<S, R>(between, lo, c0, hi, cell);
+      material(e_lo);
+      finish_cell<S, kRing, SR, X, false, unsigned>(
+          between, dst, c, 0u, mask, mid, pal, a, c, x, y, (uint8_t)m_lo, mc, cell, jout2, true,
+          seed + 1u, RecPtrs<R>{});
+    }
+    __syncwarp();   // the next first step overwrites ring row y1 - 2
+    hi = hi >= 2 * kRingCols ? hi - 2 * kRingCols : hi + kRingCols;
+    if (first) {
+      m_lo = m_hi;
+      e_lo = e_hi;
+      m_hi = m_next;
+      e_hi = e_next;
+    }
+  }
+}
+
+// Unit u of a lattice's strips x row chunks, one per warp.
+template <typename S, bool SR, bool X>
+__device__ __forceinline__ void two_steps_unit(const S *src_p, S *dst, const uint8_t *mask,
+                                               const uint16_t *mid,
+                                               const MatCoef<typename Real<S>::type> *pal,
+                                               const KArgsT<typename Real<S>::type> &a, int u,
+                                               typename Real<S>::type *jout, long long jstep) {
+  extern __shared__ __align__(16) unsigned char pair_smem[];
+  const int w = threadIdx.x >> 5, strips = (a.nx + kStripCols - 1) / kStripCols;
+  S *ring = reinterpret_cast<S *>(pair_smem) + w * (24 * kRingCells);
+  unsigned char *stage = pair_smem + kPairWarps * (24 * kRingCells * (int)sizeof(S)) + w * Stage<S>::kBytes;
+  // chunks of equal weight: a catalyst row counts two rows
+  const int chunks = (a.ny + a.ny_cl + a.pair_rows - 1) / a.pair_rows;
+  if (u >= strips * chunks) return;   // (whole warps leave)
+  // the slow units first: the end columns, then the bottom chunk upwards
+  int strip, chunk;
+  if (strips > 2) {
+    const int ends = 2 * chunks, v = u - ends, inner = strips - 2;
+    chunk = u < ends ? u >> 1 : v / inner;
+    strip = u < ends ? (u & 1) * (strips - 1) : 1 + (v - chunk * inner);
+  } else {
+    chunk = u / strips;
+    strip = u - chunk * strips;
+  }
+  auto row_at = [&](int w) { return w < 2 * a.ny_cl ? (w + 1) >> 1 : min(w - a.ny_cl, a.ny); };
+  const int ya = row_at(chunk * a.pair_rows), yb = row_at((chunk + 1) * a.pair_rows);
+  if (ya >= yb) return;
+  two_steps<S, SR, X>(src_p, dst, mask, mid, pal, a, strip, ya, yb, jout, jstep, ring, stage);
+}
+
+template <typename S, bool SR, bool X>
+__global__ void __launch_bounds__(32 * kPairWarps, pair_blocks_per_sm(sizeof(S)))
+k_step2(const S *__restrict__ src_p, S *__restrict__ dst, const uint8_t *__restrict__ mask,
+        const uint16_t *__restrict__ mid, const MatCoef<typename Real<S>::type> *__restrict__ pal,
+        KArgsT<typename Real<S>::type> a, typename Real<S>::type *__restrict__ jout,
+        long long jstep) {
+  two_steps_unit<S, SR, X>(src_p, dst, mask, mid, pal, a, blockIdx.x * kPairWarps + (threadIdx.x >> 5),
+                           jout, jstep);
 }
 
 // The step with its reverse records (plain cathode set-ups, round-to-
@@ -156,12 +379,12 @@ k_step_rec(const S *__restrict__ src_p, S *__restrict__ dst, const uint8_t *__re
   const int x = blockIdx.x * BX + (threadIdx.x % BX);
   const int y = blockIdx.y * BY + (threadIdx.x / BX);
   if (x >= a.nx || y >= a.ny) return;
-  cell_update<S, false, false, false, true>(src_p, dst, mask, mid, pal, a, x, y, rp);
+  cell_update<S, kLdg, false, false, true>(src_p, dst, mask, mid, pal, a, x, y, nullptr, rp);
 }
 
 // ------------------------------------------------------ launcher
 template <typename S, int V>
-void launch_step_v(const void *src, void *dst, const DevGeom &g, const KArgs &a, cudaStream_t st) {
+void launch_step_v(const void *src, void *dst, const DevGeom &g, const KArgs &a, void *jout, cudaStream_t st) {
   constexpr StepShape sh = kStepShapes[V];
   dim3 grid((a.nx + sh.bx - 1) / sh.bx, (a.ny + sh.by - 1) / sh.by);
   using R = typename Real<S>::type;
@@ -171,18 +394,18 @@ void launch_step_v(const void *src, void *dst, const DevGeom &g, const KArgs &a,
     constexpr StepShape sx = kStepShapes[V <= 2 ? 1 : 7];
     dim3 gx((a.nx + sx.bx - 1) / sx.bx, (a.ny + sx.by - 1) / sx.by);
     k_step<S, sx.bx, sx.by, sx.minb, false, true><<<gx, sx.bx * sx.by, 0, st>>>(
-        (const S *)src, (S *)dst, g.mask, g.mid, (const MatCoef<R> *)g.pal, narrow_args<R>(a));
+        (const S *)src, (S *)dst, g.mask, g.mid, (const MatCoef<R> *)g.pal, narrow_args<R>(a), (R *)jout);
     return;
   }
   if constexpr (sizeof(S) == 2) {
     if (a.stochastic) {
       k_step<S, sh.bx, sh.by, sh.minb, true><<<grid, sh.bx * sh.by, 0, st>>>(
-          (const S *)src, (S *)dst, g.mask, g.mid, (const MatCoef<R> *)g.pal, narrow_args<R>(a));
+          (const S *)src, (S *)dst, g.mask, g.mid, (const MatCoef<R> *)g.pal, narrow_args<R>(a), (R *)jout);
       return;
     }
   }
   k_step<S, sh.bx, sh.by, sh.minb><<<grid, sh.bx * sh.by, 0, st>>>(
-      (const S *)src, (S *)dst, g.mask, g.mid, (const MatCoef<R> *)g.pal, narrow_args<R>(a));
+      (const S *)src, (S *)dst, g.mask, g.mid, (const MatCoef<R> *)g.pal, narrow_args<R>(a), (R *)jout);
 }
 
 constexpr StepShape kRecShape = {64, 2, 6};
@@ -199,16 +422,37 @@ void launch_step_rec(const void *src, void *dst, const DevGeom &g, const KArgs &
 
 template <typename S>
 void launch_step(const void *src, void *dst, const DevGeom &g, const KArgs &a, int variant,
-                 cudaStream_t st) {
+                 void *jout, cudaStream_t st) {
   switch (variant) {
-    case 1: launch_step_v<S, 1>(src, dst, g, a, st); break;
-    case 2: launch_step_v<S, 2>(src, dst, g, a, st); break;
-    case 3: launch_step_v<S, 3>(src, dst, g, a, st); break;
-    case 4: launch_step_v<S, 4>(src, dst, g, a, st); break;
-    case 5: launch_step_v<S, 5>(src, dst, g, a, st); break;
-    case 6: launch_step_v<S, 6>(src, dst, g, a, st); break;
-    case 7: launch_step_v<S, 7>(src, dst, g, a, st); break;
-    default: launch_step_v<S, 0>(src, dst, g, a, st); break;
+    case 1: launch_step_v<S, 1>(src, dst, g, a, jout, st); break;
+    case 2: launch_step_v<S, 2>(src, dst, g, a, jout, st); break;
+    case 3: launch_step_v<S, 3>(src, dst, g, a, jout, st); break;
+    case 4: launch_step_v<S, 4>(src, dst, g, a, jout, st); break;
+    case 5: launch_step_v<S, 5>(src, dst, g, a, jout, st); break;
+    case 6: launch_step_v<S, 6>(src, dst, g, a, jout, st); break;
+    case 7: launch_step_v<S, 7>(src, dst, g, a, jout, st); break;
+    default: launch_step_v<S, 0>(src, dst, g, a, jout, st); break;
+  }
+}
+
+// Two steps: a grid of strips x row chunks (KArgsT.pair_rows).
+template <typename S, bool SR, bool X>
+void launch_step2_v(const void *src, void *dst, const DevGeom &g, const KArgs &a, void *jout,
+                    long long jstep, cudaStream_t st) {
+  using R = typename Real<S>::type;
+  k_step2<S, SR, X><<<pair_blocks(a.nx, a.ny, a.ny_cl, a.pair_rows), 32 * kPairWarps,
+                      pair_smem_bytes(sizeof(S)), st>>>(
+      (const S *)src, (S *)dst, g.mask, g.mid, (const MatCoef<R> *)g.pal, narrow_args<R>(a),
+      (R *)jout, jstep);
+}
+template <typename S>
+void launch_step2(const void *src, void *dst, const DevGeom &g, const KArgs &a, void *jout,
+                  long long jstep, cudaStream_t st) {
+  if constexpr (sizeof(S) < 8) {
+    if (needs_extended(a)) return launch_step2_v<S, false, true>(src, dst, g, a, jout, jstep, st);
+    if constexpr (sizeof(S) == 2)
+      if (a.stochastic) return launch_step2_v<S, true, false>(src, dst, g, a, jout, jstep, st);
+    launch_step2_v<S, false, false>(src, dst, g, a, jout, jstep, st);
   }
 }
 
