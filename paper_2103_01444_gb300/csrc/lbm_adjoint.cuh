@@ -21,7 +21,7 @@
 //     adjoints of x.  Catalyst cells of the volumetric mode also read their
 //     own state (through their own record); that adjoint goes to O(x).
 //     Solid cells zero their own lambda^{n-1}.
-//   k_adj_edge (one warp per listed edge cell): the same for cells with
+//   k_adj_edge (a warp per listed edge cell, eight to a block): the same for cells with
 //     boundary links, from their pulled values; the adjoint of values taken
 //     from the cell's own state goes to O(x, q), a virtual column's uses of
 //     the cells above and below to V.
@@ -544,8 +544,12 @@ __device__ __forceinline__ void adj_interior_cell(const RecPtrs<R> &rp,
 
 // Cells without edge bits, one thread per cell (grid over the lattice);
 // solid cells zero their own lambda^{n-1} (nothing is ever pushed there).
+// FP32: 128 threads at 64 registers.  FP64: single warps (two FP64 lanes per
+// SM: see kStepShapes64) with the registers it needs; at 64 registers it kept
+// 588 bytes of a thread in local memory.
+template <typename R> constexpr int adj_threads() { return sizeof(R) == 8 ? 32 : 128; }
 template <typename R>
-__global__ void __launch_bounds__(128, 8)
+__global__ void __launch_bounds__(adj_threads<R>(), sizeof(R) == 8 ? 1 : 8)
 k_adj_interior(RecPtrs<R> rp, const uint8_t *__restrict__ mask, const uint16_t *__restrict__ mid,
                const MatCoef<R> *__restrict__ pal, KArgsT<R> a, int fickian, AdjBufs<R> B) {
   const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y;
@@ -562,13 +566,17 @@ k_adj_interior(RecPtrs<R> rp, const uint8_t *__restrict__ mask, const uint16_t *
 }
 
 // Fluid cells with edge bits, one warp per entry of `cells` (linear cell
-// indices y * nxp + x), four cells per block.  An edge cell's boundary
-// pulls and their reverses are independent per link, so lane q < 24 takes
-// link q (in parallel instead of one long serial chain per cell); lane 0
-// runs the cell's collision reverse in between.  lam_complete: lambda^n
+// indices y * nxp + x), kEdgeWarps cells per block.  An edge cell's boundary
+// pulls and their reverses are independent per link, so lane q < 24 of its
+// warp takes link q (in parallel instead of one long serial chain per cell).
+// The collision reverses in between are one thread's work per cell: lane i of
+// warp 0 runs that of the block's cell i, so that one instruction serves
+// eight cells (an instruction costs the same with one lane active, and an
+// FP64 one 16 cycles of its SM; with lane 0 of every warp on its own cell
+// these instructions took as long as the whole interior).  lam_complete: lambda^n
 // holds every link in full (the seed, or the caller's), O_in and V_in are
 // zero.  seed_cell >= 0: the "CL temperature" seed on a zero lambda^n.
-constexpr int kEdgeWarps = 4, kEdgeMinBlocks = 1;
+constexpr int kEdgeWarps = 8, kEdgeMinBlocks = 1;
 // Launch order of a reverse step: the edge kernel before (true) or after
 // the interior kernel; the first one's blocks are dispatched first.
 constexpr bool kAdjEdgeFirst = true;
@@ -588,23 +596,25 @@ k_adj_edge(RecPtrs<R> rp, const uint8_t *__restrict__ mask, const uint16_t *__re
   };
   __shared__ Shared sh_all[kEdgeWarps];
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  // the cell of this thread's warp (phases 1, 3, 4)
   const int t = blockIdx.x * kEdgeWarps + w;
-  if (t >= ncells) return;   // whole warps leave
   Shared &sh = sh_all[w];
-  const long long c = cells[t], P = a.plane, W = a.nxp;
+  const long long P = a.plane;
+  bool active = t < ncells;
+  const long long c = active ? cells[t] : 0;
 #ifdef PEMLBM_BOUNDS_CHECK
   // every lambda, own-use, gradient and virtual-column access of the cell is
   // c + q P (q < 24), c itself or indexed by its row: bounded by c < P
-  if (!in_bounds(c, P, 35)) return;   // (the whole warp: one cell)
+  active = active && in_bounds(c, P, 35);   // (the whole warp: one cell)
 #endif
   const int y = (int)(c / a.nxp), x = (int)(c - (long long)y * a.nxp);
-  const uint8_t m = mask[c];
-  const MatCoef<R> mc = pal[mid[c]];
+  const uint8_t m = active ? mask[c] : (uint8_t)REG_SOLID;
+  const MatCoef<R> mc = pal[active ? mid[c] : 0];
   const bool vcol = has_vcol(a, x);
   const int vs = vcol_side(a, x);
   // ---- phase 1 (lane q): the pulled value of link q (the cell's record;
   // its slot is its index t in the list), lambda^n of link q
-  if (lane < 24) {
+  if (active && lane < 24) {
     const int q = lane;
     sh.pulled[q] = rp.pulled[24LL * t + q];
     const uint32_t pbits = lam_complete ? 0xffffffffu : B.pushed[t];
@@ -619,38 +629,49 @@ k_adj_edge(RecPtrs<R> rp, const uint8_t *__restrict__ mask, const uint16_t *__re
   }
   if (lane < 20) sh.V[lane] = R(0);
   if (lane == 0) sh.lip = sh.lw1[0] = sh.lw1[1] = sh.lw1[2] = R(0);
-  __syncwarp();
-  // ---- phase 2 (lane 0): reaction and collision reverse of the cell
+  __syncthreads();
+  // ---- phase 2 (warp 0, lane i): reaction and collision reverse of cell i
+  const int t2 = blockIdx.x * kEdgeWarps + lane;
+  bool solo = w == 0 && lane < kEdgeWarps && t2 < ncells;
+  const long long c2 = solo ? cells[t2] : 0;
+#ifdef PEMLBM_BOUNDS_CHECK
+  solo = solo && in_bounds(c2, P, 35);
+#endif
+  Shared &s2 = sh_all[lane < kEdgeWarps ? lane : 0];
+  const int y2 = (int)(c2 / a.nxp), x2 = (int)(c2 - (long long)y2 * a.nxp);
+  MatCoef<R> mc2{};
   R lphi = 0, ldarcy = 0, lforch = 0, ll0 = 0, ll1 = 0, lip = 0;
   R lb1 = 0, lq1_1 = 0, lw1[3] = {0, 0, 0};
   R gacc[3] = {0, 0, 0};
-  if (lane == 0) {
-    gacc[0] = B.gphi[c];
-    gacc[1] = B.gK[c];
-    gacc[2] = B.gD[c];
+  if (solo) {
+    const uint8_t m2 = mask[c2];
+    mc2 = pal[mid[c2]];
+    gacc[0] = B.gphi[c2];
+    gacc[1] = B.gK[c2];
+    gacc[2] = B.gD[c2];
     Cell<R> cell;
 #pragma unroll
-    for (int i = 0; i < 9; ++i) cell.f[i] = sh.pulled[i];
+    for (int i = 0; i < 9; ++i) cell.f[i] = s2.pulled[i];
 #pragma unroll
     for (int s = 0; s < 3; ++s)
 #pragma unroll
-      for (int i = 0; i < 5; ++i) cell.g[s][i] = sh.pulled[9 + 5 * s + i];
-    const bool surf = a.mode == 0 && (m & M_YLO);
-    const bool vol = a.mode == 1 && (m & REG_MASK) == REG_CATALYST;
+      for (int i = 0; i < 5; ++i) cell.g[s][i] = s2.pulled[9 + 5 * s + i];
+    const bool surf = a.mode == 0 && (m2 & M_YLO);
+    const bool vol = a.mode == 1 && (m2 & REG_MASK) == REG_CATALYST;
     R theta = 0, k = 0, ka = 0, kappa = 0, gd = 0, Cv = 0, S_vol = 0;
-    if (surf || vol) theta = rp.own[4LL * t];
+    if (surf || vol) theta = rp.own[4LL * t2];
     if (surf) {
       k = rate<R>(a, R(a.kA_surf), theta);
       ka = rate_anodic<R>(a, R(a.kA_surf_a), theta);
-      kappa = k / (R(2) * mc.w1[1]);
+      kappa = k / (R(2) * mc2.w1[1]);
       gd = cell.g[1][2] + R(a.wr1[1]) * R(a.Cref[1]);
       const R Jv = (gd * (R(2) * kappa) - ka) / (R(1) + kappa);
       cell.g[1][2] -= Jv;
-      cell.g[0][2] += R(a.hpo) * mc.inv_sigma * Jv;
+      cell.g[0][2] += R(a.hpo) * mc2.inv_sigma * Jv;
       cell.g[2][2] += R(2) * Jv;
     }
     if (vol) {
-      Cv = rp.own[4LL * t + 1];
+      Cv = rp.own[4LL * t2 + 1];
       k = rate<R>(a, R(a.kA_vol), theta);
       ka = rate_anodic<R>(a, R(a.kA_vol_a), theta);
       S_vol = (ka - k * Cv) / (R(1) + k);
@@ -660,68 +681,68 @@ k_adj_edge(RecPtrs<R> rp, const uint8_t *__restrict__ mask, const uint16_t *__re
     for (int i = 0; i < 9; ++i) lcf[i] = R(0);
     R lb[3] = {0, 0, 0}, lq1[3] = {0, 0, 0}, lsrc[3] = {0, 0, 0};
     {
-      const Macro<R> u = macros<R>(a, mc, cell);
-      const R srcv[3] = {-S_vol * R(a.hpo) * mc.inv_sigma, S_vol, R(-2) * S_vol};
+      const Macro<R> u = macros<R>(a, mc2, cell);
+      const R srcv[3] = {-S_vol * R(a.hpo) * mc2.inv_sigma, S_vol, R(-2) * S_vol};
       R lux = 0, luy = 0;
 #pragma unroll
       for (int s = 0; s < 3; ++s) {
         R lo[5];
 #pragma unroll
         for (int i = 0; i < 5; ++i) {
-          lo[i] = sh.lin[9 + 5 * s + i];
+          lo[i] = s2.lin[9 + 5 * s + i];
           lcg[s][i] = R(0);
         }
-        collide_scalar_rev<R>(a, mc, s, u.ux, u.uy, u.C[s], cell.g[s][1] - cell.g[s][3],
+        collide_scalar_rev<R>(a, mc2, s, u.ux, u.uy, u.C[s], cell.g[s][1] - cell.g[s][3],
                               cell.g[s][2] - cell.g[s][4], srcv[s], lo, lcg[s], lux, luy,
                               lsrc[s], lb[s], lw1[s], lq1[s]);
       }
       R lo[9];
 #pragma unroll
-      for (int i = 0; i < 9; ++i) lo[i] = sh.lin[i];
-      flow_rev<R>(a, mc, u.vx, u.vy, lo, lux, luy, lcf, lphi, ldarcy, lforch, ll0, ll1, lip);
+      for (int i = 0; i < 9; ++i) lo[i] = s2.lin[i];
+      flow_rev<R>(a, mc2, u.vx, u.vy, lo, lux, luy, lcf, lphi, ldarcy, lforch, ll0, ll1, lip);
     }
     if (vol) {   // volumetric sources (-S h / sigma, S, -2 S)
-      const R lS = -R(a.hpo) * mc.inv_sigma * lsrc[0] + lsrc[1] - R(2) * lsrc[2];
+      const R lS = -R(a.hpo) * mc2.inv_sigma * lsrc[0] + lsrc[1] - R(2) * lsrc[2];
       const R lC_own = lS * (-k / (R(1) + k));
       const R lth_own =
           lS * (-(Cv + ka) / ((R(1) + k) * (R(1) + k))) * drate_dtheta<R>(a, k, theta) +
           lS / (R(1) + k) * drate_anodic_dtheta<R>(a, ka, theta);
 #pragma unroll
       for (int q = 0; q < 5; ++q) {
-        sh.O[9 + q] += lth_own;
-        sh.O[14 + q] += lC_own;
+        s2.O[9 + q] += lth_own;
+        s2.O[14 + q] += lC_own;
       }
     }
-    if (c == seed_cell) {
+    if (c2 == seed_cell) {
 #pragma unroll
       for (int i = 0; i < 5; ++i) lcg[0][i] += R(1);
     }
     if (surf) {   // reverse of the surface reaction (post -> pre link values)
-      const R lJ = -lcg[1][2] + R(a.hpo) * mc.inv_sigma * lcg[0][2] + R(2) * lcg[2][2];
+      const R lJ = -lcg[1][2] + R(a.hpo) * mc2.inv_sigma * lcg[0][2] + R(2) * lcg[2][2];
       // J = (2 kappa g_d - k_a)/(1 + kappa)
       const R lgd = lJ * R(2) * kappa / (R(1) + kappa);
       const R lkap = lJ * (R(2) * gd + ka) / ((R(1) + kappa) * (R(1) + kappa));
-      const R lk = lkap / (R(2) * mc.w1[1]);
-      lw1[1] += -lkap * k / (R(2) * mc.w1[1] * mc.w1[1]);
+      const R lk = lkap / (R(2) * mc2.w1[1]);
+      lw1[1] += -lkap * k / (R(2) * mc2.w1[1] * mc2.w1[1]);
       const R lth = lk * drate_dtheta<R>(a, k, theta) +
                     (-lJ / (R(1) + kappa)) * drate_anodic_dtheta<R>(a, ka, theta);
 #pragma unroll
-      for (int q = 0; q < 5; ++q) sh.O[9 + q] += lth;
+      for (int q = 0; q < 5; ++q) s2.O[9 + q] += lth;
       lcg[1][2] += lgd;
     }
 #pragma unroll
-    for (int i = 0; i < 9; ++i) sh.lpull[i] = lcf[i];
+    for (int i = 0; i < 9; ++i) s2.lpull[i] = lcf[i];
 #pragma unroll
     for (int s = 0; s < 3; ++s)
 #pragma unroll
-      for (int i = 0; i < 5; ++i) sh.lpull[9 + 5 * s + i] = lcg[s][i];
+      for (int i = 0; i < 5; ++i) s2.lpull[9 + 5 * s + i] = lcg[s][i];
     lb1 = lb[1];
     lq1_1 = lq1[1];
   }
-  __syncwarp();
+  __syncthreads();
   // ---- phase 3 (lane q): reverse of the pull of link q
   R lU = 0;
-  if (lane < 24) {
+  if (active && lane < 24) {
     const int q = lane;
     if (q < 9) {
       pull_flow_rev<R>(rp, a, mask, mid, pal, q, x, y, m, sh.lpull[q], B.lam_out, sh.O, sh.V,
@@ -732,28 +753,30 @@ k_adj_edge(RecPtrs<R> rp, const uint8_t *__restrict__ mask, const uint16_t *__re
                          &sh.lw1[s]);
     }
   }
-  __syncwarp();
-  // ---- phase 4: own-use and virtual-column adjoints out; parameters (lane 0)
-  if (lane < 24) B.O[lane * P + c] = sh.O[lane];
-  if (vcol && lane < 10) {
+  __syncthreads();
+  // ---- phase 4: own-use and virtual-column adjoints out (lane q);
+  // parameters (warp 0, lane i)
+  if (active && lane < 24) B.O[lane * P + c] = sh.O[lane];
+  if (active && vcol && lane < 10) {
     B.V[(vs + 0 * 10 + lane) * a.ny + y] = sh.V[lane];
     B.V[(vs + 1 * 10 + lane) * a.ny + y] = sh.V[10 + lane];
   }
-  if (lane == 0) {
-    lip += sh.lip;
+  if (solo) {
+    lip += s2.lip;
 #pragma unroll
-    for (int s = 0; s < 3; ++s) lw1[s] += sh.lw1[s];
-    if (vcol) {   // the virtual column's use of this cell's 1/phi in the previous step
+    for (int s = 0; s < 3; ++s) lw1[s] += s2.lw1[s];
+    if (has_vcol(a, x2)) {   // the virtual column's use of this cell's 1/phi in the previous step
+      const int vs2 = vcol_side(a, x2);
       R vsum_ip = 0;
-      if (y + 1 < a.ny) vsum_ip += ld_r(B.V_in + (vs + 0 * 10 + 9) * a.ny + (y + 1));
-      if (y - 1 >= 0) vsum_ip += ld_r(B.V_in + (vs + 1 * 10 + 9) * a.ny + (y - 1));
-      gacc[0] += -vsum_ip * mc.inv_phi * mc.inv_phi;
+      if (y2 + 1 < a.ny) vsum_ip += ld_r(B.V_in + (vs2 + 0 * 10 + 9) * a.ny + (y2 + 1));
+      if (y2 - 1 >= 0) vsum_ip += ld_r(B.V_in + (vs2 + 1 * 10 + 9) * a.ny + (y2 - 1));
+      gacc[0] += -vsum_ip * mc2.inv_phi * mc2.inv_phi;
     }
-    param_rev<R>(a, mc, fickian, lphi, ldarcy, lforch, ll0, ll1, lip, lb1, lw1[1], lq1_1,
+    param_rev<R>(a, mc2, fickian, lphi, ldarcy, lforch, ll0, ll1, lip, lb1, lw1[1], lq1_1,
                  &gacc[0], &gacc[1], &gacc[2]);
-    B.gphi[c] = gacc[0];
-    B.gK[c] = gacc[1];
-    B.gD[c] = gacc[2];
+    B.gphi[c2] = gacc[0];
+    B.gK[c2] = gacc[1];
+    B.gD[c2] = gacc[2];
   }
   // inlet drive (velocity, or dp_in): warp sum, one FP64 atomic per warp that has inlet links
 #pragma unroll

@@ -592,8 +592,9 @@ void launch_adj_step(const RecBufs &r, const DevGeom &g, const KArgs &a, int fic
   };
   if (b.n_edge > 0) cudaEventRecord(fork, st);
   if (kAdjEdgeFirst) edge();
-  k_adj_interior<R><<<dim3((a.nx + 127) / 128, a.ny), 128, 0, st>>>(rp, g.mask, g.mid, pal, an,
-                                                                    fickian, B);
+  constexpr int T = adj_threads<R>();
+  k_adj_interior<R><<<dim3((a.nx + T - 1) / T, a.ny), T, 0, st>>>(rp, g.mask, g.mid, pal, an, fickian,
+                                                                  B);
   if (!kAdjEdgeFirst) edge();
   if (b.n_edge > 0) cudaStreamWaitEvent(st, join, 0);
 }
