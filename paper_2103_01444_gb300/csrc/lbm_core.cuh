@@ -1013,8 +1013,17 @@ __device__ __forceinline__ Macro<R> macros(const KArgsT<R> &a, const MatCoef<R> 
   if constexpr (X) vy += R(0.5) * mc.phi * Gy;
   // u = v / den with one reciprocal of den; |u| = |v| / den, so u's
   // magnitude needs no square root of its own
-  R vn = vsqrt(vx * vx + vy * vy);
-  R inv_den = vrcp(mc.l0 + vsqrt(mc.l0 * mc.l0 + mc.l1 * vn));
+  R vn, inv_den;
+  if (sizeof(R) == 8 && mc.l1 == R(0)) {
+    // clear fluid, or Darcy drag alone: the denominator is 2 l0 exactly and
+    // |u| is multiplied by forch = 0.  FP64 has two lanes per SM, and the two
+    // roots and the division are a fifth of a cell's FP64 instructions.
+    vn = R(0);
+    inv_den = mc.l0 == R(0.5) ? R(1) : R(0.5) / mc.l0;
+  } else {
+    vn = vsqrt(vx * vx + vy * vy);
+    inv_den = vrcp(mc.l0 + vsqrt(mc.l0 * mc.l0 + mc.l1 * vn));
+  }
   r.vx = vx;
   r.vy = vy;
   r.ux = vx * inv_den;
@@ -1087,10 +1096,12 @@ __device__ __forceinline__ void collide_flow(const KArgsT<R> &a, const MatCoef<R
 }
 
 // D2Q5 MRT collision of scalar s in deviation moments (Eq. 10), plus a
-// volumetric source src added with the cell's equilibrium weights.
+// volumetric source src added with the cell's equilibrium weights (react:
+// whether it can be non-zero).
 template <typename R>
 __device__ __forceinline__ void collide_scalar(const KArgsT<R> &a, const MatCoef<R> &mc, int s,
-                                               R ux, R uy, R Cdev, const R d[5], R srcv, R o[5]) {
+                                               R ux, R uy, R Cdev, const R d[5], R srcv, R o[5],
+                                               bool react) {
   const R Q1 = mc.q1[s], Q3 = R(a.Q3);
   // the advected value: C, or its excess over the inlet value (then about
   // zero in the deviation storage, so the flux populations stay small)
@@ -1111,13 +1122,23 @@ __device__ __forceinline__ void collide_scalar(const KArgsT<R> &a, const MatCoef
   // collision conserves C up to one local rounding (5 * 0.2 != 1 in binary:
   // the scaled form would multiply every cell's C by the same factor at
   // every step)
-  R ev = n0 * R(0.2) + n3 * R(0.05) + w1 * srcv;
+  R ev, n0s = n0;
+  if (sizeof(R) == 8) {   // (FP64 instructions are dear: none for cells without a source)
+    ev = n0 * R(0.2) + n3 * R(0.05);
+    if (react) {
+      ev += w1 * srcv;
+      n0s += srcv;
+    }
+  } else {
+    ev = n0 * R(0.2) + n3 * R(0.05) + w1 * srcv;
+    n0s = n0 + srcv;
+  }
   R ex = ev + R(0.25) * n4, ey = ev - R(0.25) * n4;
   o[1] = ex + R(0.5) * n1;
   o[3] = ex - R(0.5) * n1;
   o[2] = ey + R(0.5) * n2;
   o[4] = ey - R(0.5) * n2;
-  o[0] = (n0 + srcv) - ((o[1] + o[3]) + (o[2] + o[4]));
+  o[0] = n0s - ((o[1] + o[3]) + (o[2] + o[4]));
 }
 
 }  // namespace pemlbm

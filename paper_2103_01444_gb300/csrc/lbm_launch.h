@@ -36,6 +36,13 @@ constexpr int pair_blocks_per_sm(size_t esize) { return esize == 4 ? 8 : 10; }
 // a lattice's blocks.
 int pair_rows(const int *nx, const int *ny, const int *ny_cl, int n, size_t esize);
 int pair_blocks(int nx, int ny, int ny_cl, int rows);
+// The FP64 step is bound by the two FP64 lanes of an SM (a warp instruction
+// takes 16 cycles), so its warps are spread over all SMs: with the 128 x 2
+// blocks of the other types a 250 x 64 lattice used 64 of the 152 SMs (27.8 us
+// a step, now 16.2).  Default 128 threads, 32 x 4.
+constexpr StepShape kStepShapes64[kStepVariants] = {
+    {32, 4, 1}, {64, 1, 1}, {32, 2, 1}, {128, 1, 1}, {32, 1, 1}, {64, 2, 1}, {128, 2, 1}, {256, 1, 1}};
+constexpr StepShape step_shape(size_t esize, int v) { return esize == 8 ? kStepShapes64[v] : kStepShapes[v]; }
 constexpr int kReduceThreads = 512;
 // Persistent batched step: 128 x 1 cells per block, 8 blocks per SM asked of
 // the register allocator; the grid is the number of co-resident blocks.

@@ -155,7 +155,7 @@ __device__ __forceinline__ void finish_cell(const Pops<S, CG> &src, S *__restric
   R g[3][5];
 #pragma unroll
   for (int s = 0; s < 3; ++s)
-    collide_scalar<R>(a, mc, s, u.ux, u.uy, u.C[s], cell.g[s], srcv[s], g[s]);
+    collide_scalar<R>(a, mc, s, u.ux, u.uy, u.C[s], cell.g[s], srcv[s], g[s], S_vol != R(0));
   if (live) {   // links 0-4 of the flow and the three scalars, one group each
 #pragma unroll
     for (int i = 0; i < 5; ++i) {
@@ -192,6 +192,40 @@ __device__ __forceinline__ void cell_update(const S *__restrict__ src_p, S *__re
                                             cell, jout, true, seed, rp);
 }
 
+// The cell of a thread in blocks of BX x BY cells.  FP64: the first blocks
+// walk up the two end columns and the others cover the columns between.  An
+// FP64 instruction costs the same with one active lane as with 32, and the
+// boundary links of the ends (inlet parabola, the outlet's virtual column)
+// are almost as many as a cell's own: in row blocks every row paid for them
+// twice, now each 32 rows do.  (509 x 127: 44.4 -> 40 us a step, 1024 x
+// 256: 140 -> 136; 250 x 64, bound by a warp's latency, 16.2 both ways.)
+template <typename S, int BX, int BY>
+__device__ __forceinline__ bool cell_of_thread(int nx, int ny, int &x, int &y) {
+  if constexpr (sizeof(S) == 8) {
+    constexpr int T = BX * BY;
+    const int per_end = (ny + T - 1) / T;
+    int b = blockIdx.x;
+    if (b < 2 * per_end) {
+      x = b < per_end ? 0 : nx - 1;
+      y = (b < per_end ? b : b - per_end) * T + threadIdx.x;
+      return y < ny;
+    }
+    b -= 2 * per_end;
+    const int across = (nx - 2 + BX - 1) / BX;
+    x = 1 + b % across * BX + threadIdx.x % BX;
+    y = b / across * BY + threadIdx.x / BX;
+    return x < nx - 1 && y < ny;
+  } else {
+    x = blockIdx.x * BX + threadIdx.x % BX;
+    y = blockIdx.y * BY + threadIdx.x / BX;
+    return x < nx && y < ny;
+  }
+}
+inline dim3 ends_first_grid(int nx, int ny, StepShape sh) {
+  const int T = sh.bx * sh.by;
+  return dim3(2 * ((ny + T - 1) / T) + (nx - 2 + sh.bx - 1) / sh.bx * ((ny + sh.by - 1) / sh.by));
+}
+
 // SR: 16-bit stores with stochastic rounding (a separate instantiation, so
 // the round-to-nearest kernel carries none of its code); X as cell_update.
 template <typename S, int BX, int BY, int MINB, bool SR = false, bool X = false>
@@ -199,9 +233,8 @@ __global__ void __launch_bounds__(BX * BY, MINB)
 k_step(const S *__restrict__ src_p, S *__restrict__ dst, const uint8_t *__restrict__ mask,
        const uint16_t *__restrict__ mid, const MatCoef<typename Real<S>::type> *__restrict__ pal,
        KArgsT<typename Real<S>::type> a, typename Real<S>::type *__restrict__ jout) {
-  const int x = blockIdx.x * BX + (threadIdx.x % BX);
-  const int y = blockIdx.y * BY + (threadIdx.x / BX);
-  if (x >= a.nx || y >= a.ny) return;
+  int x, y;
+  if (!cell_of_thread<S, BX, BY>(a.nx, a.ny, x, y)) return;
   cell_update<S, kLdg, SR, X>(src_p, dst, mask, mid, pal, a, x, y, jout);
 }
 
@@ -385,14 +418,17 @@ k_step_rec(const S *__restrict__ src_p, S *__restrict__ dst, const uint8_t *__re
 // ------------------------------------------------------ launcher
 template <typename S, int V>
 void launch_step_v(const void *src, void *dst, const DevGeom &g, const KArgs &a, void *jout, cudaStream_t st) {
-  constexpr StepShape sh = kStepShapes[V];
+  constexpr StepShape sh = step_shape(sizeof(S), V);
   dim3 grid((a.nx + sh.bx - 1) / sh.bx, (a.ny + sh.by - 1) / sh.by);
+  if (sizeof(S) == 8) grid = ends_first_grid(a.nx, a.ny, sh);
   using R = typename Real<S>::type;
   if (needs_extended(a)) {
     // two shapes of the extended step: 128 x 2 at 80 registers (variants
-    // 0-2) and 64 x 2 at 64 registers (the rest); the tuner picks one
-    constexpr StepShape sx = kStepShapes[V <= 2 ? 1 : 7];
+    // 0-2) and 64 x 2 at 64 registers (the rest); the tuner picks one (FP64:
+    // 64 x 1 and 256 x 1)
+    constexpr StepShape sx = step_shape(sizeof(S), V <= 2 ? 1 : 7);
     dim3 gx((a.nx + sx.bx - 1) / sx.bx, (a.ny + sx.by - 1) / sx.by);
+    if (sizeof(S) == 8) gx = ends_first_grid(a.nx, a.ny, sx);
     k_step<S, sx.bx, sx.by, sx.minb, false, true><<<gx, sx.bx * sx.by, 0, st>>>(
         (const S *)src, (S *)dst, g.mask, g.mid, (const MatCoef<R> *)g.pal, narrow_args<R>(a), (R *)jout);
     return;
@@ -408,15 +444,16 @@ void launch_step_v(const void *src, void *dst, const DevGeom &g, const KArgs &a,
       (const S *)src, (S *)dst, g.mask, g.mid, (const MatCoef<R> *)g.pal, narrow_args<R>(a), (R *)jout);
 }
 
-constexpr StepShape kRecShape = {64, 2, 6};
+// (FP64: see kStepShapes64)
+template <typename S> constexpr StepShape kRecShape = sizeof(S) == 8 ? StepShape{32, 1, 1} : StepShape{64, 2, 6};
 template <typename S>
 void launch_step_rec(const void *src, void *dst, const DevGeom &g, const KArgs &a,
                      const RecBufs &r, cudaStream_t st) {
   using R = typename Real<S>::type;
-  dim3 grid((a.nx + kRecShape.bx - 1) / kRecShape.bx, (a.ny + kRecShape.by - 1) / kRecShape.by);
+  constexpr StepShape sh = kRecShape<S>;
+  dim3 grid((a.nx + sh.bx - 1) / sh.bx, (a.ny + sh.by - 1) / sh.by);
   const RecPtrs<R> rp{(R *)r.cell, (R *)r.own, (R *)r.pulled, r.slot};
-  k_step_rec<S, kRecShape.bx, kRecShape.by, kRecShape.minb><<<grid, kRecShape.bx * kRecShape.by,
-                                                              0, st>>>(
+  k_step_rec<S, sh.bx, sh.by, sh.minb><<<grid, sh.bx * sh.by, 0, st>>>(
       (const S *)src, (S *)dst, g.mask, g.mid, (const MatCoef<R> *)g.pal, narrow_args<R>(a), rp);
 }
 
