@@ -135,7 +135,8 @@ struct lbm_domain {
   double *hsmall = nullptr;    // pinned host mirror
   double *scratch = nullptr;   // [24][ny][nx] doubles, lazily allocated
   void *pal_scratch = nullptr; // device palette build's work space, allocated at its first use
-  float *dprofile = nullptr;   // [nx]
+  float *hprofile = nullptr;   // pinned host [nx]: the local current as the kernel writes it
+  unsigned *ddone = nullptr;   // finished blocks of the catalyst reduction (0 between calls)
   // references of the deviation storage: part of the state's representation,
   // so they change only at reset (or with a loaded state)
   double Cref[3] = {0, 0, 0}, bref[3] = {0, 0, 0};
@@ -561,7 +562,8 @@ lbm_status lbm_create_domain(const lbm_domain_desc *desc, lbm_domain **out) {
       dmalloc(&d->colsum, sizeof(double) * 2 * d->nx) != cudaSuccess ||
       dmalloc(&d->dsmall, sizeof(double) * 16) != cudaSuccess || dmalloc(&d->dbad, sizeof(int)) != cudaSuccess ||
       dmalloc(&d->dseed, 256) != cudaSuccess ||
-      dmalloc(&d->dprofile, sizeof(float) * d->nx) != cudaSuccess ||
+      dmalloc(&d->ddone, sizeof(unsigned)) != cudaSuccess ||
+      hmalloc(&d->hprofile, sizeof(float) * d->nx) != cudaSuccess ||
       hmalloc(&d->hsmall, sizeof(double) * 16) != cudaSuccess) {
     cudaGetLastError();
     return cleanup(fail(LBM_ENOMEM, "device allocation of %.1f MB failed", 2.0 * pop_bytes / 1e6));
@@ -573,6 +575,7 @@ lbm_status lbm_create_domain(const lbm_domain_desc *desc, lbm_domain **out) {
     if (dmalloc(&dsolid, (size_t)D.nx * D.ny) != cudaSuccess) return cleanup(fail(LBM_ENOMEM, "solid mask"));
     cudaMemcpyAsync(dsolid, D.solid, (size_t)D.nx * D.ny, cudaMemcpyHostToDevice, d->stream);
   }
+  cudaMemsetAsync(d->ddone, 0, sizeof(unsigned), d->stream);
   cudaMemsetAsync(d->mid, 0, cells * 2, d->stream);
   cudaMemsetAsync(d->pop[0], 0, pop_bytes, d->stream);
   cudaMemsetAsync(d->pop[1], 0, pop_bytes, d->stream);
@@ -591,10 +594,11 @@ lbm_status lbm_destroy_domain(lbm_domain *d) {
   drop_graphs(d);
   for (void *p : {d->pop[0], d->pop[1], (void *)d->mask, (void *)d->mid, d->pal, (void *)d->raw,
                   d->snap, (void *)d->partial, (void *)d->colsum, (void *)d->dsmall, (void *)d->dbad, (void *)d->dseed,
-                  (void *)d->scratch, (void *)d->dprofile, (void *)d->dobs, d->jcells, (void *)d->jcol,
+                  (void *)d->scratch, (void *)d->ddone, (void *)d->dobs, d->jcells, (void *)d->jcol,
                   d->pal_scratch})
     if (p) cudaFree(p);
   if (d->hsmall) cudaFreeHost(d->hsmall);
+  if (d->hprofile) cudaFreeHost(d->hprofile);
   if (d->hobs) cudaFreeHost(d->hobs);
   for (auto e : {d->obs_done[0], d->obs_done[1]})
     if (e) cudaEventDestroy(e);
@@ -877,13 +881,12 @@ lbm_status lbm_current_density(lbm_domain *d, double *i_avg, double *heat, float
   const KArgs a = make_args(d);
   dispatch(d->desc.precision, [&](auto *tag) {
     using S = std::remove_pointer_t<decltype(tag)>;
-    launch_catalyst<S>(d->pop[d->cur ^ 1], geom(d), a, i_scale, profile ? d->dprofile : nullptr,
-                       d->colsum, d->dsmall, d->stream);
+    launch_catalyst<S>(d->pop[d->cur ^ 1], geom(d), a, i_scale, profile ? d->hprofile : nullptr,
+                       d->colsum, d->hsmall, d->ddone, d->stream);
   });
   CK(cudaGetLastError());
-  CK(cudaMemcpyAsync(d->hsmall, d->dsmall, 2 * sizeof(double), cudaMemcpyDeviceToHost, d->stream));
-  if (profile) CK(cudaMemcpyAsync(profile, d->dprofile, sizeof(float) * d->nx, cudaMemcpyDeviceToHost, d->stream));
-  CK(cudaStreamSynchronize(d->stream));
+  CK(cudaStreamSynchronize(d->stream));   // the kernel wrote the pinned results
+  if (profile) std::memcpy(profile, d->hprofile, sizeof(float) * d->nx);
   if (i_avg) *i_avg = d->hsmall[0] * i_scale / d->nx;
   if (heat) *heat = d->hsmall[1] * q_scale / d->nx;
   return LBM_OK;
@@ -943,7 +946,7 @@ lbm_status lbm_balances(lbm_domain *d, double *out) {
   dispatch(d->desc.precision, [&](auto *tag) {
     using S = std::remove_pointer_t<decltype(tag)>;
     launch_catalyst<S>(d->pop[d->cur ^ 1], geom(d), a, 1.0, nullptr, d->colsum, d->dsmall,
-                       d->stream);
+                       d->ddone, d->stream);
     launch_balances<S>(d->pop[d->cur ^ 1], geom(d), a, d->dsmall + 2, d->stream);
   });
   CK(cudaGetLastError());
@@ -1591,7 +1594,7 @@ lbm_status lbm_grad(lbm_domain *d, int32_t objective, int64_t nsteps, int32_t se
     const double i_scale = 4.0 * p.F * p.c_tot * p.dx_cm / p.dt_s;
     dispatch(d->desc.precision, [&](auto *tag) {
       using S = std::remove_pointer_t<decltype(tag)>;
-      launch_catalyst<S>(sN1, g, a, i_scale, nullptr, d->colsum, d->dsmall, d->stream);
+      launch_catalyst<S>(sN1, g, a, i_scale, nullptr, d->colsum, d->dsmall, d->ddone, d->stream);
       launch_adj_seed_current<S>(sN1, g, a, d->prm.interface_mode == 1, i_scale / d->nx,
                                  w.ptrs(1), d->stream);   // writes lam[0]
     });

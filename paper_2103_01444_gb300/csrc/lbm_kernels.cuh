@@ -272,12 +272,16 @@ k_balances(const S *__restrict__ src_p, const uint8_t *__restrict__ mask,
 // sum of the volumetric sinks over the catalyst rows) is reduced in shared
 // memory in a fixed order and written, with its heat h J(x), to colsum
 // [2][nx] (FP64); profile[x] = J(x) i_scale (A/cm^2) when not NULL.
+// The block that finishes last (done counts them and is left at 0) sums the
+// columns into out[0], out[1] in the order of k_sum_columns: one launch, and
+// out and profile may be pinned host memory, so a reading call waits for one
+// kernel instead of two and two copies (200 x 40: 32.7 -> 20.3 us).
 template <typename S>
 __global__ void __launch_bounds__(kCatalystBX * kCatalystBY)
 k_catalyst(const S *__restrict__ src_p, const uint8_t *__restrict__ mask,
            const uint16_t *__restrict__ mid, const MatCoef<typename Real<S>::type> *__restrict__ pal,
            KArgsT<typename Real<S>::type> a, double i_scale, float *__restrict__ profile,
-           double *__restrict__ colsum) {
+           double *colsum, double *__restrict__ out, unsigned *__restrict__ done) {
   using R = typename Real<S>::type;
   __shared__ double sm[kCatalystBY][kCatalystBX];
   const Pops<S> src{src_p, a.plane, a.nxp};
@@ -308,6 +312,43 @@ k_catalyst(const S *__restrict__ src_p, const uint8_t *__restrict__ mask,
     colsum[x] = t;
     colsum[a.nx + x] = t * a.hpo;
     if (profile) profile[x] = (float)(t * i_scale);
+  }
+  __shared__ bool last;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) last = atomicAdd(done, 1u) == gridDim.x - 1;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  // thread t stands for the threads t and t + T of k_sum_columns
+  constexpr int T = kCatalystBX * kCatalystBY, W = kReduceThreads / 32;
+  static_assert(2 * T == kReduceThreads, "two column strides per thread");
+  __shared__ double part[2 * 32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    double acc[2] = {0.0, 0.0};
+    for (int c = threadIdx.x + h * T; c < a.nx; c += kReduceThreads) {
+      acc[0] += __ldcg(colsum + c);
+      acc[1] += __ldcg(colsum + a.nx + c);
+    }
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+#pragma unroll
+      for (int off = 16; off > 0; off >>= 1) acc[k] += __shfl_down_sync(0xffffffffu, acc[k], off);
+      if (lane == 0) part[k * 32 + warp + h * (W / 2)] = acc[k];
+    }
+  }
+  __syncthreads();
+  if (warp == 0) {
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      double t = lane < W ? part[k * 32 + lane] : 0.0;
+#pragma unroll
+      for (int off = 16; off > 0; off >>= 1) t += __shfl_down_sync(0xffffffffu, t, off);
+      if (lane == 0) out[k] = t;
+    }
+    if (lane == 0) *done = 0u;
   }
 }
 
@@ -658,12 +699,11 @@ void launch_balances(const void *src, const DevGeom &g, const KArgs &a, double *
 
 template <typename S>
 void launch_catalyst(const void *src, const DevGeom &g, const KArgs &a, double i_scale,
-                     float *profile, double *colsum, double *out, cudaStream_t st) {
+                     float *profile, double *colsum, double *out, unsigned *done, cudaStream_t st) {
   const int nb = (a.nx + kCatalystBX - 1) / kCatalystBX;
   k_catalyst<S><<<nb, kCatalystBX * kCatalystBY, 0, st>>>(
       (const S *)src, g.mask, g.mid, (const MatCoef<typename Real<S>::type> *)g.pal,
-      narrow_args<typename Real<S>::type>(a), i_scale, profile, colsum);
-  k_sum_columns<<<1, kReduceThreads, 0, st>>>(colsum, a.nx, out);
+      narrow_args<typename Real<S>::type>(a), i_scale, profile, colsum, out, done);
 }
 
 template <typename S>
@@ -721,7 +761,7 @@ template <typename S> unsigned long long bounds_first_bad() {
   template void launch_balances<S>(const void *, const DevGeom &, const KArgs &, double *,      \
                                    cudaStream_t);                                                \
   template void launch_catalyst<S>(const void *, const DevGeom &, const KArgs &, double,        \
-                                   float *, double *, double *, cudaStream_t);                  \
+                                   float *, double *, double *, unsigned *, cudaStream_t);      \
   template void launch_residual<S>(const void *, const DevGeom &, const KArgs &, const void *,  \
                                    void *, double *, int *, double *, cudaStream_t);            \
   template void launch_init<S>(void *, const DevGeom &, const KArgs &, cudaStream_t);           \

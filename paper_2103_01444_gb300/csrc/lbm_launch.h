@@ -78,7 +78,7 @@ struct RecBufs {
 template <typename S> void launch_step_rec(const void *src, void *dst, const DevGeom &g, const KArgs &a, const RecBufs &r, cudaStream_t st);
 template <typename S> void launch_fields(const void *src, const DevGeom &g, const KArgs &a, double *out, cudaStream_t st);
 template <typename S> void launch_balances(const void *src, const DevGeom &g, const KArgs &a, double *out, cudaStream_t st);
-template <typename S> void launch_catalyst(const void *src, const DevGeom &g, const KArgs &a, double i_scale, float *profile, double *colsum, double *out, cudaStream_t st);
+template <typename S> void launch_catalyst(const void *src, const DevGeom &g, const KArgs &a, double i_scale, float *profile, double *colsum, double *out, unsigned *done, cudaStream_t st);
 // (J, heat) of nsteps observed steps from what their cells consumed
 // ([step][rows][nx], arithmetic precision) into out [step][2].
 void launch_sum_reaction(const void *jcells, bool fp64, int nx, int rows, int nsteps, double hpo, double *colsum, double *out, cudaStream_t st);
