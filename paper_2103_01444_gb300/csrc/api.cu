@@ -158,6 +158,10 @@ struct lbm_domain {
   bool halo_lo = false, halo_hi = false;
   std::vector<uint8_t> hsolid;                 // the whole lattice's solids (slabs)
   cudaEvent_t ev_halo = nullptr;
+  // reverse workspace of lbm_grad and lbm_vjp, kept between calls when small
+  // (adj_work)
+  void *adj = nullptr;
+  void (*adj_free)(void *) = nullptr;
 };
 
 namespace {
@@ -592,6 +596,7 @@ lbm_status lbm_destroy_domain(lbm_domain *d) {
   if (!d) return LBM_OK;
   if (d->stream) cudaStreamSynchronize(d->stream);
   drop_graphs(d);
+  if (d->adj) d->adj_free(d->adj);
   for (void *p : {d->pop[0], d->pop[1], (void *)d->mask, (void *)d->mid, d->pal, (void *)d->raw,
                   d->snap, (void *)d->partial, (void *)d->colsum, (void *)d->dsmall, (void *)d->dbad, (void *)d->dseed,
                   (void *)d->scratch, (void *)d->ddone, (void *)d->dobs, d->jcells, (void *)d->jcol,
@@ -1192,7 +1197,8 @@ struct DevBuf {
 
 // Reverse workspace of one domain.
 struct AdjWork {
-  DevBuf lam[2], O[2], V[2], gphi, gK, gD, gU, tphi, tK, tD, cells, pushed, slot;
+  DevBuf lam[2], O[2], V[2], gphi, gK, gD, gU, tphi, tK, tD, cells, pushed, slot, fs[2];
+  size_t bytes = 0;                             // of the lattice-sized buffers
   int n_edge = 0, n_own = 0;
   size_t rsize = 4;                             // bytes of the arithmetic type
   cudaStream_t side = nullptr;                  // edge-cell branch of each step
@@ -1215,11 +1221,12 @@ struct AdjWork {
       if ((s = b->alloc(planes * r)) != LBM_OK) return s;
     for (auto *b : {&V[0], &V[1]})   // [outlet, inlet][down, up][10][ny]
       if ((s = b->alloc(40 * (size_t)d->ny * r)) != LBM_OK) return s;
-    // everything starts at zero: lambda^{n-1} of solid cells is zeroed by
-    // every step, and the own-use parts of the first lambda are zero
-    for (auto *b : {&lam[0], &lam[1], &O[0], &O[1]})
-      CK(cudaMemsetAsync(b->p, 0, planes * r, d->stream));
-    for (auto *b : {&V[0], &V[1]}) CK(cudaMemsetAsync(b->p, 0, 40 * (size_t)d->ny * r, d->stream));
+    // forward states, with the guard of a domain's buffers
+    const size_t sbytes = (24 * (size_t)d->plane + d->nxp + 64) * d->esize;
+    for (auto &b : fs)
+      if ((s = b.alloc(sbytes)) != LBM_OK) return s;
+    bytes = 4 * planes * r + 2 * sbytes + 3 * (r + sizeof(double)) * (size_t)d->plane +
+            sizeof(int) * (size_t)d->plane;
     for (auto *b : {&gphi, &gK, &gD})
       if ((s = b->alloc(r * d->plane)) != LBM_OK) return s;
     for (auto *b : {&tphi, &tK, &tD})
@@ -1304,8 +1311,13 @@ struct AdjWork {
     return RecBufs{b, b + rec_cell_bytes(d), b + rec_cell_bytes(d) + rec_own_bytes(),
                    (const int *)slot.p};
   }
-  lbm_status zero_grads(const lbm_domain *d) {
-    const size_t r = fp64(d) ? 8 : 4;
+  // The start of a reverse sweep: gradients, and everything a first step
+  // adds to or reads beside the seed, at zero (lambda^{n-1} of solid cells is
+  // zeroed by every step, the own-use parts of the first lambda are zero).
+  lbm_status begin(const lbm_domain *d) {
+    const size_t r = fp64(d) ? 8 : 4, planes = 24 * (size_t)d->plane;
+    for (auto *b : {&lam[0], &lam[1], &O[0], &O[1]}) CK(cudaMemsetAsync(b->p, 0, planes * r, d->stream));
+    for (auto *b : {&V[0], &V[1]}) CK(cudaMemsetAsync(b->p, 0, 40 * (size_t)d->ny * r, d->stream));
     for (auto *b : {&gphi, &gK, &gD}) CK(cudaMemsetAsync(b->p, 0, r * d->plane, d->stream));
     for (auto *b : {&tphi, &tK, &tD}) CK(cudaMemsetAsync(b->p, 0, sizeof(double) * d->plane, d->stream));
     CK(cudaMemsetAsync(gU.p, 0, sizeof(double), d->stream));
@@ -1325,6 +1337,38 @@ struct AdjWork {
     b.lam = nullptr;
     b.O_in = b.V_in = nullptr;
     return b;   // lam_out = lam[cur], O = O[cur], V = V[cur]
+  }
+};
+
+// The reverse workspace of a domain for one call.  Its allocations, the cell
+// lists built on the host and the matching frees took 1.9 ms of every call
+// (1024 x 256), so it stays with the domain until that is destroyed where it
+// is below 1/64 of the device's memory, and is released after the call beyond
+// that.
+struct AdjLease {
+  lbm_domain *d = nullptr;
+  AdjWork *w = nullptr;
+  bool keep = false;
+  ~AdjLease() {
+    if (!w || keep) return;
+    cudaStreamSynchronize(d->stream);
+    delete w;
+    d->adj = nullptr;
+  }
+  lbm_status take(lbm_domain *dom) {
+    d = dom;
+    size_t free_b = 0, total_b = 0;
+    if (!d->adj) {
+      w = new AdjWork();
+      lbm_status s = w->alloc(d);
+      if (s != LBM_OK) return s;
+      d->adj = w;
+      d->adj_free = [](void *p) { delete (AdjWork *)p; };
+    }
+    w = (AdjWork *)d->adj;
+    CK(cudaMemGetInfo(&free_b, &total_b));
+    keep = w->bytes <= total_b / 64;
+    return w->begin(d);
   }
 };
 
@@ -1440,9 +1484,9 @@ lbm_status lbm_vjp(lbm_domain *d, const double *lam_next, double *lam_prev, doub
   if (!lam_next || !lam_prev) return fail(LBM_EINVAL, "null argument");
   if (d->desc.rounding != 0) return fail(LBM_EINVAL, "the adjoint needs round-to-nearest storage");
   if ((s = adjoint_covers(d)) != LBM_OK) return s;
-  AdjWork w;
-  if ((s = w.alloc(d)) != LBM_OK) return s;
-  if ((s = w.zero_grads(d)) != LBM_OK) return s;
+  AdjLease lease;
+  if ((s = lease.take(d)) != LBM_OK) return s;
+  AdjWork &w = *lease.w;
   if ((s = lam_upload(d, lam_next, w.lam[0].p)) != LBM_OK) return s;
   // the step's reverse records (its new state is not kept)
   DevBuf rec, next;
@@ -1476,13 +1520,11 @@ lbm_status lbm_grad(lbm_domain *d, int32_t objective, int64_t nsteps, int32_t se
   const int seg = segment > 0 ? segment : (int)std::ceil(std::sqrt((double)N));
   const int64_t nseg = (nrec + seg - 1) / seg;   // segment k: R^{k seg + 1} .. R^{min((k+1) seg, nrec)}
   const size_t sbytes = (24 * (size_t)d->plane + d->nxp + 64) * d->esize;   // guard as in the domain
-  AdjWork w;
-  if ((s = w.alloc(d)) != LBM_OK) return s;
-  if ((s = w.zero_grads(d)) != LBM_OK) return s;
+  AdjLease lease;
+  if ((s = lease.take(d)) != LBM_OK) return s;
+  AdjWork &w = *lease.w;
+  DevBuf(&fs)[2] = w.fs;   // forward states
   const size_t rbytes = w.rec_bytes(d), segbytes = rbytes * (size_t)seg;
-  DevBuf fs[2];   // forward states
-  for (auto &b : fs)
-    if ((s = b.alloc(sbytes)) != LBM_OK) return s;
   // The last L segments keep the records their forward steps write; the
   // others are recomputed from checkpoints (two record buffers, so that
   // segment k - 1 is recomputed on a stream of its own while segment k is
