@@ -535,9 +535,10 @@ lbm_status lbm_create_domain(const lbm_domain_desc *desc, lbm_domain **out) {
   d->nxp = (need + align - 1) / align * align;
   d->plane = (long long)d->nxp * D.ny;
   d->esize = elem_size(D.precision);
-  // untuned default: 64 x 2 cells at 8 blocks per SM for FP32 storage (the
-  // tuner's usual choice at large sizes), the uncapped 128 x 2 otherwise
-  d->variant = D.precision == LBM_FP32 ? 7 : 0;
+  // untuned default: 64 x 2 cells at 8 blocks per SM (the tuner's usual choice
+  // at large sizes: 8192 x 2048 grains with stochastic FP16 433 us a step, 623
+  // with the uncapped 128 x 2); FP64 has shapes of its own
+  d->variant = fp64(d) ? 0 : 7;
   d->pair_rows = pair_rows(&d->nx, &d->ny, &D.ny_cl, 1, d->esize);
   auto cleanup = [&](lbm_status s) { lbm_destroy_domain(d); return s; };
   cudaError_t allowed = cudaSuccess;

@@ -126,11 +126,27 @@ __device__ __forceinline__ float ld_s(const __half *p) { return __half2float(*p)
 __device__ __forceinline__ unsigned short sr_bits(const __nv_bfloat16 *, float v, unsigned r16) {
   return (unsigned short)((__float_as_uint(v) + r16) >> 16);
 }
-__device__ __forceinline__ unsigned short sr_bits(const __half *, float v, unsigned r16) {
+// v plus that uniform fraction, ready for FP16's conversion toward zero.
+// (The integer to float conversion runs on a pipe that is idle otherwise;
+// building r16 / 65536 in a mantissa costs the full ones more: 468 against
+// 433 us a step at 8192 x 2048.)
+__device__ __forceinline__ float sr_half_sum(float v, unsigned r16) {
   const unsigned e = __float_as_uint(v) & 0x7f800000u;
   const float spacing = __uint_as_float(max(e, 113u << 23) - (10u << 23));
-  const float a = fmaf(copysignf(spacing, v), (float)r16 * (1.0f / 65536.0f), v);
-  return __half_as_ushort(__float2half_rz(a));
+  return fmaf(copysignf(spacing, v), (float)r16 * (1.0f / 65536.0f), v);
+}
+__device__ __forceinline__ unsigned short sr_bits(const __half *, float v, unsigned r16) {
+  return __half_as_ushort(__float2half_rz(sr_half_sum(v, r16)));
+}
+// Two values as one word, the first in the low half.
+__device__ __forceinline__ unsigned sr_pair(const __nv_bfloat16 *, float a, float b, unsigned ra,
+                                            unsigned rb) {
+  return __byte_perm(__float_as_uint(a) + ra, __float_as_uint(b) + rb, 0x7632);
+}
+__device__ __forceinline__ unsigned sr_pair(const __half *, float a, float b, unsigned ra, unsigned rb) {
+  unsigned r;
+  asm("cvt.rz.f16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(sr_half_sum(b, rb)), "f"(sr_half_sum(a, ra)));
+  return r;
 }
 template <typename S> __device__ __forceinline__ void st_sr(S *p, float v, unsigned r16) {
   *reinterpret_cast<unsigned short *>(p) = sr_bits(p, v, r16);
@@ -214,10 +230,6 @@ __device__ __forceinline__ void stq(double *p, double a, double b, double c, dou
   reinterpret_cast<double2 *>(p)[0] = make_double2(a, b);
   reinterpret_cast<double2 *>(p)[1] = make_double2(c, d);
 }
-__device__ __forceinline__ uint2 pack4(unsigned short a, unsigned short b, unsigned short c,
-                                       unsigned short d) {
-  return make_uint2((unsigned)a | ((unsigned)b << 16), (unsigned)c | ((unsigned)d << 16));
-}
 // (paired conversions: each half rounds as __float2bfloat16_rn / __float2half_rn)
 __device__ __forceinline__ void stq(__nv_bfloat16 *p, float a, float b, float c, float d) {
   const __nv_bfloat162 lo = __floats2bfloat162_rn(a, b), hi = __floats2bfloat162_rn(c, d);
@@ -234,8 +246,7 @@ __device__ __forceinline__ void stq(__half *p, float a, float b, float c, float 
 template <typename S>
 __device__ __forceinline__ void stq_sr(S *p, float a, float b, float c, float d, unsigned ra,
                                        unsigned rb, unsigned rc, unsigned rd) {
-  *reinterpret_cast<uint2 *>(p) =
-      pack4(sr_bits(p, a, ra), sr_bits(p, b, rb), sr_bits(p, c, rc), sr_bits(p, d, rd));
+  *reinterpret_cast<uint2 *>(p) = make_uint2(sr_pair(p, a, b, ra, rb), sr_pair(p, c, d, rc, rd));
 }
 
 // Material coefficients of one palette entry, derived from (phi, K, alpha)
@@ -415,6 +426,15 @@ template <typename S, int CG = kLdg> struct Pops {
 #endif
     return ldp<CG>(p + pop_index(q, (long long)y * nxp + x, plane));
   }
+  // the group of link i (flow, T, O2, H2O)
+  __device__ __forceinline__ auto group(int i, int x, int y) const {
+#ifdef PEMLBM_BOUNDS_CHECK
+    const long long k = pop_index(i, (long long)y * nxp + x, plane);
+    using V = decltype(ldq<CG>(p));
+    if (!in_bounds(k, pop_extent(plane, nxp), 1) || !in_bounds(k + 3, pop_extent(plane, nxp), 1)) return V{};
+#endif
+    return ldq<CG>(p + pop_index(i, (long long)y * nxp + x, plane));
+  }
 };
 
 // The row ring that a warp of the two-step kernel (k_step2) keeps in shared
@@ -434,6 +454,13 @@ template <typename S> struct Pops<S, kRing> {
     if (!in_bounds(x - x_lo, kRingCols, 5)) return V(0);
 #endif
     return ld_s(p + (int)pop_index(q, c, kRingCells));
+  }
+  __device__ __forceinline__ auto group(int i, int x, int y) const {
+#ifdef PEMLBM_BOUNDS_CHECK
+    using V = decltype(ldq_s(p));
+    if (!in_bounds(x - x_lo, kRingCols, 5)) return V{};
+#endif
+    return ldq_s(p + 4 * (i * kRingCells + row(y) + x - x_lo));
   }
 };
 
@@ -805,14 +832,19 @@ template <typename S, typename R, int CG = kLdg>
 __device__ __forceinline__ void bounce_solid(const Pops<S, CG> &src, int x, int y, uint32_t nb,
                                              Cell<R> &c) {
   const int OP[9] = OP9_TAB;
+  // an axis link's four values come back in one group load
 #pragma unroll
-  for (int i = 1; i < 9; ++i)
+  for (int i = 1; i < 5; ++i)
+    if (nb & (1u << (i - 1))) {
+      const auto q = src.group(OP[i], x, y);
+      c.f[i] = q.v[0];
+      c.g[0][i] = q.v[1];
+      c.g[1][i] = q.v[2];
+      c.g[2][i] = q.v[3];
+    }
+#pragma unroll
+  for (int i = 5; i < 9; ++i)
     if (nb & (1u << (i - 1))) c.f[i] = R(src.at(OP[i], x, y));
-#pragma unroll
-  for (int s = 0; s < 3; ++s)
-#pragma unroll
-    for (int i = 1; i < 5; ++i)
-      if (nb & (1u << (i - 1))) c.g[s][i] = R(src.at(9 + 5 * s + OP[i], x, y));
 }
 
 // Replaces the pulls of links that cross a wall, the inlet, the outlet, a
@@ -879,9 +911,10 @@ __device__ __forceinline__ void fix_edges(const Pops<S, CG> &src, const KArgsT<R
   if (m & M_XLO) {   // links 1, 5, 8; the D2Q5 link 1
     const int in[3] = {1, 5, 8}, op[3] = {3, 7, 6}, ey[3] = {0, 1, -1};
     const bool open = (m & M_INLET) != 0;
+    const auto q = src.group(3, x, y);
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-      R w = R(src.at(op[k], x, y));
+      R w = k == 0 ? R(q.v[0]) : R(src.at(op[k], x, y));
       if (open && !a.inlet_pressure)
         w += R(6) * w9<R>(in[k]) * R(1) * inlet_u<R>(a, R(y) - R(0.5) * R(ey[k]));
       c.f[in[k]] = w;
@@ -893,7 +926,7 @@ __device__ __forceinline__ void fix_edges(const Pops<S, CG> &src, const KArgsT<R
     }
 #pragma unroll
     for (int s = 0; s < 3; ++s) {
-      R w = R(src.at(9 + 5 * s + 3, x, y));
+      R w = R(q.v[1 + s]);
       if (open) {
         w = wall_value<R>(a, mc, s, w, R(a.Cin[s]));
       } else if constexpr (X) {
@@ -905,43 +938,46 @@ __device__ __forceinline__ void fix_edges(const Pops<S, CG> &src, const KArgsT<R
   if (m & M_XHI) {   // links 3, 6, 7; the D2Q5 link 3
     const int in[3] = {3, 6, 7}, op[3] = {1, 8, 5}, ey[3] = {0, 1, -1};
     const bool closed = X && a.closed_x;
+    const auto q = src.group(closed ? 1 : 3, x, y);
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
       const int sy = y - ey[k];
-      if (closed) c.f[in[k]] = R(src.at(op[k], x, y));
+      if (closed) c.f[in[k]] = k == 0 ? R(q.v[0]) : R(src.at(op[k], x, y));
       else if (sy >= 0 && sy < a.ny)
         c.f[in[k]] = virtual_link<S, R, CG>(src, a, mid, pal, in[k], x, sy, R(0));
     }
 #pragma unroll
     for (int s = 0; s < 3; ++s) {
       if (closed) {
-        R w = R(src.at(9 + 5 * s + 1, x, y));
+        R w = R(q.v[1 + s]);
         if ((a.wall_dir >> (3 + s)) & 1) w = wall_value<R>(a, mc, s, w, R(a.Cwall[1][s]));
         c.g[s][3] = w;
       } else {
-        c.g[s][3] = R(src.at(9 + 5 * s + 3, x, y));   // fully developed
+        c.g[s][3] = R(q.v[1 + s]);   // fully developed
       }
     }
   }
   if (m & M_YLO) {   // links 2, 5, 6: the bottom wall
-    c.f[2] = R(src.at(4, x, y));
+    const auto q = src.group(4, x, y);
+    c.f[2] = R(q.v[0]);
     c.f[5] = R(src.at(7, x, y));
     c.f[6] = R(src.at(8, x, y));
 #pragma unroll
     for (int s = 0; s < 3; ++s) {
-      R w = R(src.at(9 + 5 * s + 4, x, y));
+      R w = R(q.v[1 + s]);
       if constexpr (X)
         if ((a.wall_dir >> (6 + s)) & 1) w = wall_value<R>(a, mc, s, w, R(a.Cwall[2][s]));
       c.g[s][2] = w;
     }
   }
   if (m & M_YHI) {   // links 4, 7, 8: the top wall
-    c.f[4] = R(src.at(2, x, y));
+    const auto q = src.group(2, x, y);
+    c.f[4] = R(q.v[0]);
     c.f[7] = R(src.at(5, x, y));
     c.f[8] = R(src.at(6, x, y));
 #pragma unroll
     for (int s = 0; s < 3; ++s) {
-      R w = R(src.at(9 + 5 * s + 2, x, y));
+      R w = R(q.v[1 + s]);
       if (a.top_dirichlet) w = wall_value<R>(a, mc, s, w, R(a.Ctop[s]));
       c.g[s][4] = w;
     }
