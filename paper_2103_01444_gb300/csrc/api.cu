@@ -129,10 +129,10 @@ struct lbm_domain {
   int variant = 0;             // launch shape of the step kernel (lbm_tune picks one)
   int64_t grad_mem_limit = -1; // device bytes lbm_grad may keep records in (-1: what is free)
   double tuned_ms[kStepVariants] = {};
-  double *dsmall = nullptr;    // device results (16 doubles)
+  double *dsmall = nullptr;    // device results (16 doubles), then ddone
   int *dbad = nullptr;
   unsigned *dseed = nullptr;   // step counter seeding stochastic 16-bit rounding
-  double *hsmall = nullptr;    // pinned host mirror
+  double *hsmall = nullptr;    // pinned host mirror, then hprofile
   double *scratch = nullptr;   // [24][ny][nx] doubles, lazily allocated
   void *pal_scratch = nullptr; // device palette build's work space, allocated at its first use
   float *hprofile = nullptr;   // pinned host [nx]: the local current as the kernel writes it
@@ -287,19 +287,31 @@ bool can_pair(const lbm_domain *d) {
          d->plane * 4 * (long long)d->esize < (1LL << 32);
 }
 
-// How n steps are launched: pairs of steps, then single steps.  A run that
-// ends with a single step (`open` false) leaves the state before its last
-// step in the other buffer, where the read-outs of that step look for it.
+// Whether four steps may run as one launch (k_step4): where pairs may, on
+// lattices of at most eight of its blocks per SM.  us a step in pairs and in
+// fours, FP32: 200 x 40 (32 blocks) 3.5, 2.0; 640 x 160 (400) 5.9, 4.1; 1024 x
+// 256 (1040) 10.0, 8.5; 1300 x 320 (1600) 12.6, 12.8.
+bool can_quad(const lbm_domain *d) {
+  const long long blocks = (long long)((d->nx + kQuadCols - 1) / kQuadCols) * ((d->ny + kQuadRows - 1) / kQuadRows);
+  return can_pair(d) && blocks <= 8 * 152;
+}
+
+// How n steps are launched: four at a time, pairs, then single steps.  A run
+// that ends with a single step (`open` false) leaves the state before its
+// last step in the other buffer, where the read-outs of that step look for
+// it.
 struct StepPlan {
-  int64_t pairs, singles;
-  int64_t launches() const { return pairs + singles; }
+  int64_t quads, pairs, singles;
+  int64_t launches() const { return quads + pairs + singles; }
+  int steps(int64_t launch) const { return launch < quads ? 4 : launch < quads + pairs ? 2 : 1; }
 };
-StepPlan plan_steps(const lbm_domain *d, int64_t n, bool open) {
-  StepPlan p{0, n};
-  if (can_pair(d)) {
-    p.pairs = open ? n / 2 : (n > 0 ? (n - 1) / 2 : 0);
-    p.singles = n - 2 * p.pairs;
-  }
+StepPlan plan_steps(bool quad, bool pair, int64_t n, bool open) {
+  StepPlan p{0, 0, open || n == 0 ? 0 : 1};
+  int64_t left = n - p.singles;
+  if (quad) p.quads = left / 4;
+  left -= 4 * p.quads;
+  if (pair) p.pairs = left / 2;
+  p.singles += left - 2 * p.pairs;
   return p;
 }
 
@@ -314,16 +326,18 @@ lbm_status launch_plan(lbm_domain *d, const KArgs &a, StepPlan plan, int cur, in
   };
   int64_t step = 0;
   for (int64_t k = 0; k < plan.launches(); ++k) {
-    const bool pair = k < plan.pairs;
+    const int n = plan.steps(k);
     dispatch(d->desc.precision, [&](auto *tag) {
       using S = std::remove_pointer_t<decltype(tag)>;
-      if (pair)
+      if (n == 4)
+        launch_step4<S>(d->pop[cur], d->pop[cur ^ 1], g, a, slot(step), jstep, st);
+      else if (n == 2)
         launch_step2<S>(d->pop[cur], d->pop[cur ^ 1], g, a, slot(step), jstep, st);
       else
         launch_step<S>(d->pop[cur], d->pop[cur ^ 1], g, a, variant, slot(step), st);
     });
-    if (a.stochastic) launch_seed_advance(d->dseed, pair ? 2 : 1, st);
-    step += pair ? 2 : 1;
+    if (a.stochastic) launch_seed_advance(d->dseed, n, st);
+    step += n;
     cur ^= 1;
   }
   CK(cudaGetLastError());
@@ -332,7 +346,7 @@ lbm_status launch_plan(lbm_domain *d, const KArgs &a, StepPlan plan, int cur, in
 
 lbm_status launch_steps(lbm_domain *d, int64_t n, bool open = false, void *jout = nullptr,
                         int64_t jstep = 0) {
-  const StepPlan plan = plan_steps(d, n, open);
+  const StepPlan plan = plan_steps(can_quad(d), can_pair(d), n, open);
   lbm_status s = launch_plan(d, make_args(d), plan, d->cur, d->variant, jout, jstep, d->stream);
   if (s == LBM_OK) d->cur ^= (int)(plan.launches() & 1);
   return s;
@@ -565,14 +579,14 @@ lbm_status lbm_create_domain(const lbm_domain_desc *desc, lbm_domain **out) {
       dmalloc(&d->snap, 2 * rsize * 5 * (size_t)d->nx * D.ny) != cudaSuccess ||
       dmalloc(&d->partial, sizeof(double) * 10 * residual_blocks(d->nx, D.ny)) != cudaSuccess ||
       dmalloc(&d->colsum, sizeof(double) * 2 * d->nx) != cudaSuccess ||
-      dmalloc(&d->dsmall, sizeof(double) * 16) != cudaSuccess || dmalloc(&d->dbad, sizeof(int)) != cudaSuccess ||
+      dmalloc(&d->dsmall, sizeof(double) * 17) != cudaSuccess || dmalloc(&d->dbad, sizeof(int)) != cudaSuccess ||
       dmalloc(&d->dseed, 256) != cudaSuccess ||
-      dmalloc(&d->ddone, sizeof(unsigned)) != cudaSuccess ||
-      hmalloc(&d->hprofile, sizeof(float) * d->nx) != cudaSuccess ||
-      hmalloc(&d->hsmall, sizeof(double) * 16) != cudaSuccess) {
+      hmalloc(&d->hsmall, sizeof(double) * 16 + sizeof(float) * d->nx) != cudaSuccess) {
     cudaGetLastError();
     return cleanup(fail(LBM_ENOMEM, "device allocation of %.1f MB failed", 2.0 * pop_bytes / 1e6));
   }
+  d->ddone = (unsigned *)(d->dsmall + 16);
+  d->hprofile = (float *)(d->hsmall + 16);
   if (cudaEventCreate(&d->ev0) != cudaSuccess || cudaEventCreate(&d->ev1) != cudaSuccess)
     return cleanup(fail(LBM_ECUDA, "cudaEventCreate failed"));
   uint8_t *dsolid = nullptr;
@@ -600,11 +614,10 @@ lbm_status lbm_destroy_domain(lbm_domain *d) {
   if (d->adj) d->adj_free(d->adj);
   for (void *p : {d->pop[0], d->pop[1], (void *)d->mask, (void *)d->mid, d->pal, (void *)d->raw,
                   d->snap, (void *)d->partial, (void *)d->colsum, (void *)d->dsmall, (void *)d->dbad, (void *)d->dseed,
-                  (void *)d->scratch, (void *)d->ddone, (void *)d->dobs, d->jcells, (void *)d->jcol,
+                  (void *)d->scratch, (void *)d->dobs, d->jcells, (void *)d->jcol,
                   d->pal_scratch})
     if (p) cudaFree(p);
   if (d->hsmall) cudaFreeHost(d->hsmall);
-  if (d->hprofile) cudaFreeHost(d->hprofile);
   if (d->hobs) cudaFreeHost(d->hobs);
   for (auto e : {d->obs_done[0], d->obs_done[1]})
     if (e) cudaEventDestroy(e);
@@ -1802,7 +1815,8 @@ lbm_status batch_lanes(lbm_batch *b, int64_t n, bool fixed_parity, bool open) {
     // trials: the same launch again and again, two steps' worth each
     const bool pair = can_pair(d);
     const int64_t reps = fixed_parity ? (pair ? n : 2 * n) : 1;
-    const StepPlan plan = !fixed_parity ? plan_steps(d, n, open) : pair ? StepPlan{1, 0} : StepPlan{0, 1};
+    const StepPlan plan = !fixed_parity ? plan_steps(false, pair, n, open)
+                          : StepPlan{0, pair ? 1 : 0, pair ? 0 : 1};
     for (int64_t k = 0; k < reps; ++k) {
       lbm_status s = launch_plan(d, a, plan, d->cur, b->variant, nullptr, 0, b->lanes[c]);
       if (s != LBM_OK) return s;
@@ -1876,13 +1890,13 @@ lbm_status batch_join_out(lbm_batch *b) {
 
 // The launches of n steps of schedule 0: all cases alike.
 StepPlan batch_plan(const lbm_batch *b, int64_t n, bool open) {
-  return b->pairs ? plan_steps(b->doms[0], n, open) : StepPlan{0, n};
+  return plan_steps(false, b->pairs, n, open);
 }
 void batch_launch_plan(lbm_batch *b, StepPlan plan) {
   for (int64_t k = 0; k < plan.launches(); ++k)
     dispatch(b->precision, [&](auto *tag) {
       using S = std::remove_pointer_t<decltype(tag)>;
-      if (k < plan.pairs)
+      if (plan.steps(k) == 2)
         launch_batch_step2<S>(b->dcases, b->dpair, (int)b->doms.size(), b->pair_blocks, (int)(k & 1),
                               b->stream);
       else
@@ -1990,7 +2004,7 @@ lbm_status batch_run(lbm_batch *b, int64_t nsteps, bool fixed_parity) {
   if ((s = batch_table(b, sh.bx)) != LBM_OK) return s;
   if (fixed_parity) {   // trials of two steps each, as batch_lanes
     for (int64_t k = 0; k < (b->pairs ? nsteps : 2 * nsteps); ++k)
-      batch_launch_plan(b, b->pairs ? StepPlan{1, 0} : StepPlan{0, 1});
+      batch_launch_plan(b, StepPlan{0, b->pairs ? 1 : 0, b->pairs ? 0 : 1});
     CK(cudaGetLastError());
     return LBM_OK;
   }
@@ -2179,9 +2193,11 @@ lbm_status lbm_batch_tune(lbm_batch *b, int32_t trial_steps, int32_t *schedule, 
     }
     return LBM_OK;
   };
-  for (int v = 0; v < kStepVariants && s == LBM_OK; ++v) s = trial(0, v);
+  // (in pairs the shape matters only to a run's last step or two)
+  const int first = b->pairs ? kStepVariants - 1 : 0;
+  for (int v = first; v < kStepVariants && s == LBM_OK; ++v) s = trial(0, v);
   if (s == LBM_OK) s = trial(1, 6);
-  for (int v = 0; v < kStepVariants && s == LBM_OK; ++v) s = trial(3, v);
+  for (int v = first; v < kStepVariants && s == LBM_OK; ++v) s = trial(3, v);
   // the trials wrote each case's next state into its other buffer: restore
   for (lbm_domain *d : b->doms) {
     const KArgs a = make_args(d);

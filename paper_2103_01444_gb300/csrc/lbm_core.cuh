@@ -72,9 +72,9 @@ enum : uint8_t {
 
 // --------------------------------------------------------------- storage
 // Where a kernel reads populations from: a global buffer through the
-// read-only path, a global buffer past L1, or the row ring that the
-// two-step kernel keeps in shared memory (Pops).
-enum : int { kLdg = 0, kLdcg = 1, kRing = 2 };
+// read-only path, a global buffer past L1, the row ring that the two-step
+// kernel keeps in shared memory, or the four-step kernel's tile there (Pops).
+enum : int { kLdg = 0, kLdcg = 1, kRing = 2, kTile = 3 };
 template <typename S> struct Real { using type = float; };
 template <> struct Real<double> { using type = double; };
 
@@ -464,6 +464,30 @@ template <typename S> struct Pops<S, kRing> {
   }
 };
 
+// The tile of the four-step kernel (k_step4): kTileWarps rows of 32 columns,
+// one row per warp, laid out like a population buffer whose planes are the
+// tile.
+constexpr int kTileWarps = 16, kTileCells = 32 * kTileWarps;
+template <typename S> struct Pops<S, kTile> {
+  const S *p;
+  int x_lo, y_lo;
+  __device__ __forceinline__ int cell(int x, int y) const { return (y - y_lo) * 32 + x - x_lo; }
+  __device__ __forceinline__ auto at(int q, int x, int y) const {
+#ifdef PEMLBM_BOUNDS_CHECK
+    using V = decltype(ld_s(p));
+    if (!in_bounds(x - x_lo, 32, 6) || !in_bounds(y - y_lo, kTileWarps, 6)) return V(0);
+#endif
+    return ld_s(p + (int)pop_index(q, cell(x, y), kTileCells));
+  }
+  __device__ __forceinline__ auto group(int i, int x, int y) const {
+#ifdef PEMLBM_BOUNDS_CHECK
+    using V = decltype(ldq_s(p));
+    if (!in_bounds(x - x_lo, 32, 6) || !in_bounds(y - y_lo, kTileWarps, 6)) return V{};
+#endif
+    return ldq_s(p + 4 * (i * kTileCells + cell(x, y)));
+  }
+};
+
 // Inlet parabola at height yh (cell centres at integer y).
 template <typename R> __device__ __forceinline__ R inlet_u(const KArgsT<R> &a, R yh) {
   R s = (yh - R(a.y_ch0) + R(0.5)) / R(a.h_ch);
@@ -771,12 +795,11 @@ __device__ __forceinline__ void take_interior(int lane, const unsigned char *sta
 }
 
 // The same from the row ring, given the ring cells lo, c0, hi of the cell
-// below, the cell itself and the cell above.  (Ring column 0 and the last
-// have no neighbour on one side and are not pulled into.)
-template <typename S, typename R>
-__device__ __forceinline__ void load_interior(const Pops<S, kRing> &src, int lo, int c0, int hi,
-                                              Cell<R> &c) {
-  constexpr int P = kRingCells;
+// below, the cell itself and the cell above, or from the tile.  (Columns and
+// rows without a neighbour on one side are not pulled into.)
+template <int CG, typename S, typename R>
+__device__ __forceinline__ void load_shared(const Pops<S, CG> &src, int lo, int c0, int hi, Cell<R> &c) {
+  constexpr int P = CG == kRing ? kRingCells : kTileCells;
   const int from[5] = {c0, c0 - 1, lo, c0 + 1, hi};
 #pragma unroll
   for (int i = 0; i < 5; ++i) {
@@ -900,7 +923,7 @@ __device__ __forceinline__ void fix_edges(const Pops<S, CG> &src, const KArgsT<R
                                           const MatCoef<R> *__restrict__ pal,
                                           const MatCoef<R> &mc, int x, int y, uint8_t m,
                                           Cell<R> &c) {
-  if constexpr (CG != kRing)
+  if constexpr (CG < kRing)
     if (a.periodic) {
       fix_links<S, R, CG, X>(src, a, mask, mid, pal, mc, x, y, m, c);
       return;

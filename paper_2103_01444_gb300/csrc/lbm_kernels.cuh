@@ -560,7 +560,8 @@ void launch_batch_step2(const BatchCase *cases, const int *block_start, int ncas
         (const BatchCaseT<typename Real<S>::type> *)cases, block_start, ncases, parity);
 }
 
-// Opts the two-step kernels into their shared memory on the current device.
+// Opts the kernels of several steps into their shared memory on the current
+// device.
 template <typename S>
 cudaError_t allow_step2() {
   if constexpr (sizeof(S) < 8) {
@@ -571,6 +572,9 @@ cudaError_t allow_step2() {
     if constexpr (sizeof(S) == 2)
       if (e == cudaSuccess) e = cudaFuncSetAttribute(k_step2<S, true, false>, attr, n);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_batch_step2<S>, attr, n);
+    const int n4 = (int)quad_smem_bytes(sizeof(S));
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_step4<S, false>, attr, n4);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_step4<S, true>, attr, n4);
     return e;
   }
   return cudaSuccess;
@@ -754,6 +758,8 @@ template <typename S> unsigned long long bounds_first_bad() {
   template void launch_step<S>(const void *, void *, const DevGeom &, const KArgs &, int,       \
                                void *, cudaStream_t);                                           \
   template void launch_step2<S>(const void *, void *, const DevGeom &, const KArgs &, void *,    \
+                                long long, cudaStream_t);                                       \
+  template void launch_step4<S>(const void *, void *, const DevGeom &, const KArgs &, void *,    \
                                 long long, cudaStream_t);                                       \
   template cudaError_t allow_step2<S>();                                                   \
   template void launch_fields<S>(const void *, const DevGeom &, const KArgs &, double *,        \

@@ -32,6 +32,10 @@ constexpr size_t pair_smem_bytes(size_t esize) {
   return (size_t)kPairWarps * (96 * 24 * esize + 32 * (esize == 4 ? 24 : 20) * esize);
 }
 constexpr int pair_blocks_per_sm(size_t esize) { return esize == 4 ? 8 : 10; }
+// Shape of the four-step kernel: blocks of 16 warps, a row of 32 columns each,
+// that finish kQuadCols x kQuadRows cells; two tiles of shared memory.
+constexpr int kQuadCols = 26, kQuadRows = 10;
+constexpr size_t quad_smem_bytes(size_t esize) { return 2 * 24 * 512 * esize; }
 // Weighted rows of a unit's chunk for one lattice or the cases of a batch, and
 // a lattice's blocks.
 int pair_rows(const int *nx, const int *ny, const int *ny_cl, int n, size_t esize);
@@ -66,6 +70,7 @@ struct DevGeom {
 };
 
 template <typename S> void launch_step(const void *src, void *dst, const DevGeom &g, const KArgs &a, int variant, void *jout, cudaStream_t st);
+template <typename S> void launch_step4(const void *src, void *dst, const DevGeom &g, const KArgs &a, void *jout, long long jstep, cudaStream_t st);
 template <typename S> cudaError_t allow_step2();
 template <typename S> void launch_step2(const void *src, void *dst, const DevGeom &g, const KArgs &a, void *jout, long long jstep, cudaStream_t st);
 // Reverse records of one step (device pointers, the arithmetic type of the

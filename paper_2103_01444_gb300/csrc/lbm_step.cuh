@@ -345,7 +345,7 @@ __device__ __forceinline__ void two_steps(const S *__restrict__ src_p, S *__rest
       const int lo = hi >= 2 * kRingCols ? hi - 2 * kRingCols : hi + kRingCols;
       const int c0 = hi >= kRingCols ? hi - kRingCols : hi + 2 * kRingCols;
       Cell<R> cell;
-      load_interior<S, R>(between, lo, c0, hi, cell);
+      load_shared(between, lo, c0, hi, cell);
       material(e_lo);
       finish_cell<S, kRing, SR, X, false, unsigned>(
           between, dst, c, 0u, mask, mid, pal, a, c, x, y, (uint8_t)m_lo, mc, cell, jout2, true,
@@ -400,6 +400,62 @@ k_step2(const S *__restrict__ src_p, S *__restrict__ dst, const uint8_t *__restr
         long long jstep) {
   two_steps_unit<S, SR, X>(src_p, dst, mask, mid, pal, a, blockIdx.x * kPairWarps + (threadIdx.x >> 5),
                            jout, jstep);
+}
+
+// ------------------------------------------------------- four steps (K1c)
+// Four steps of a small lattice: each warp takes one row of 32 columns through
+// four steps in shared memory, and every step gives up a column and a row on
+// each side, so a block finishes kQuadCols x kQuadRows cells (62% of its
+// work).  Small lattices are bound by the latency of a cell's dependent
+// instructions (about 1.6 us) and of a launch; here four steps pay for one
+// launch, one load from the L2 cache and four times that latency, where
+// k_step2's warps walk four rows in turn for two steps.  200 x 40, FP32: 2.0
+// us a step against 3.5 in pairs and 6.9 one by one (can_quad: where the
+// repeated work outweighs it).
+template <typename S, bool X>
+__global__ void __launch_bounds__(32 * kTileWarps, 1)
+k_step4(const S *__restrict__ src_p, S *__restrict__ dst, const uint8_t *__restrict__ mask,
+        const uint16_t *__restrict__ mid, const MatCoef<typename Real<S>::type> *__restrict__ pal,
+        KArgsT<typename Real<S>::type> a, typename Real<S>::type *__restrict__ jout,
+        long long jstep) {
+  using R = typename Real<S>::type;
+  extern __shared__ __align__(16) unsigned char quad_smem[];
+  S *const buf = reinterpret_cast<S *>(quad_smem);   // two tiles
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int x_lo = blockIdx.x * kQuadCols - 3, y_lo = blockIdx.y * kQuadRows - 3;
+  const int x = x_lo + lane, y = y_lo + w, k = w * 32 + lane;
+  const bool in = x >= 0 && x < a.nx && y >= 0 && y < a.ny;
+  const bool own = in && lane >= 3 && lane < 3 + kQuadCols && w >= 3 && w < 3 + kQuadRows;
+  const unsigned c = (unsigned)y * (unsigned)a.nxp + (unsigned)x;
+  uint8_t m = REG_SOLID;
+  MatCoef<R> mc{};
+  Cell<R> cell;
+  if (in) {
+    const Pops<S, kLdg> src{src_p, a.plane, a.nxp};
+    m = ld_mask(mask, c, a, 20);
+    load_interior<S, R, kLdg>(src, a, x, y, cell);
+    mc = pal[ld_mid(mid, c, a, 21)];
+    finish_cell<S, kLdg, false, X, false, int>(src, buf, k, kTileCells, mask, mid, pal, a, c, x, y, m, mc,
+                                               cell, jout, own, 0u, RecPtrs<R>{});
+  }
+  for (int t = 1; t < 3; ++t) {
+    __syncthreads();
+    const Pops<S, kTile> tile{buf + (t == 1 ? 0 : 24 * kTileCells), x_lo, y_lo};
+    if (in && lane >= t && lane < 32 - t && w >= t && w < kTileWarps - t) {
+      load_shared(tile, k - 32, k, k + 32, cell);
+      finish_cell<S, kTile, false, X, false, int>(
+          tile, buf + (t == 1 ? 24 * kTileCells : 0), k, kTileCells, mask, mid, pal, a, c, x, y, m, mc, cell,
+          jout ? jout + t * jstep : nullptr, own, 0u, RecPtrs<R>{});
+    }
+  }
+  __syncthreads();
+  if (own) {
+    const Pops<S, kTile> tile{buf, x_lo, y_lo};
+    load_shared(tile, k - 32, k, k + 32, cell);
+    finish_cell<S, kTile, false, X, false, unsigned>(tile, dst, c, 0u, mask, mid, pal, a, c, x, y, m, mc, cell,
+                                                     jout ? jout + 3 * jstep : nullptr, true, 0u,
+                                                     RecPtrs<R>{});
+  }
 }
 
 // The step with its reverse records (plain cathode set-ups, round-to-
@@ -490,6 +546,19 @@ void launch_step2(const void *src, void *dst, const DevGeom &g, const KArgs &a, 
     if constexpr (sizeof(S) == 2)
       if (a.stochastic) return launch_step2_v<S, true, false>(src, dst, g, a, jout, jstep, st);
     launch_step2_v<S, false, false>(src, dst, g, a, jout, jstep, st);
+  }
+}
+
+template <typename S>
+void launch_step4(const void *src, void *dst, const DevGeom &g, const KArgs &a, void *jout,
+                  long long jstep, cudaStream_t st) {
+  if constexpr (sizeof(S) < 8) {
+    using R = typename Real<S>::type;
+    const dim3 grid((a.nx + kQuadCols - 1) / kQuadCols, (a.ny + kQuadRows - 1) / kQuadRows);
+    auto kern = needs_extended(a) ? k_step4<S, true> : k_step4<S, false>;
+    kern<<<grid, 32 * kTileWarps, quad_smem_bytes(sizeof(S)), st>>>(
+        (const S *)src, (S *)dst, g.mask, g.mid, (const MatCoef<R> *)g.pal, narrow_args<R>(a), (R *)jout,
+        jstep);
   }
 }
 

@@ -1,6 +1,6 @@
-"""Two steps in one launch: runs that take their steps two at a time must
-leave the states, read-outs and observed reactions of single steps, bit for
-bit."""
+"""Several steps in one launch: runs that take their steps two or four at a
+time must leave the states, read-outs and observed reactions of single steps,
+bit for bit."""
 import numpy as np
 import pytest
 
@@ -11,15 +11,19 @@ pytestmark = pytest.mark.gpu
 
 def set_ups():
     """Lattices around the strips of 30 columns and the chunks of rows of the
-    two-step kernel, with every kind of boundary link."""
+    two-step kernel and the 26 x 10 blocks of the four-step one, with every kind
+    of boundary link; the last ones have too many blocks for four at a time."""
     out = []
-    for nx, ny in ((30, 24), (31, 25), (29, 61), (61, 26), (200, 40), (331, 97)):
+    for nx, ny in ((30, 24), (31, 25), (26, 61), (53, 30), (200, 40), (331, 97)):
         out.append(("film", W.small_cathode(nx, ny, 0, Re=3.0)))
         out.append(("rows", W.small_cathode(nx, ny, 1, Re=3.0)))
     out.append(("grains", W.small_cathode(152, 64, 0, grains=True)))
     out.append(("pressure", dict(W.small_cathode(140, 31, 1), inlet="pressure", dp_in=5e-4)))
     out.append(("anodic", dict(W.small_cathode(140, 31, 0), alpha_a=0.5, V_op=1.0, scalar_advection=1)))
+    out.append(("long", W.cathode_blocks(3001, 120, Re=3.0)))
+    out.append(("long", W.small_cathode(2610, 127, 0, Re=3.0, grains=True, random_material=False)))
     out.append(("cavity", W.natural_convection_cavity(95, heated_bottom=True)))
+    out.append(("cavity", W.natural_convection_cavity(601)))
     out.append(("kang", W.kang_surface_reaction(97, 48)))
     return out
 
@@ -27,7 +31,7 @@ def set_ups():
 @pytest.mark.parametrize("precision,rounding", [("fp32", "nearest"), ("bf16", "nearest"),
                                                 ("fp16", "nearest"), ("fp16", "stochastic"),
                                                 ("bf16", "stochastic"), ("fp64", "nearest")])
-@pytest.mark.parametrize("n", [2, 3, 22])
+@pytest.mark.parametrize("n", [2, 5, 22])
 def test_pairs_equal_single_steps(precision, rounding, n):
     from paper_2103_01444_gb300.build import build
     from paper_2103_01444_gb300.lbm import Domain
