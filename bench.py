@@ -222,15 +222,35 @@ class ClockSampler:
                 "samples": len(sm)}
 
 
+def steps_per_pass(precision, rounding="nearest"):
+    """Steps that one pass over the populations takes on these lattices: the
+    library runs two per launch (k_step2) except in FP64 and with stochastic
+    rounding."""
+    return 1 if precision == "fp64" or rounding != "nearest" else 2
+
+
+def observed_launches(n, pairs):
+    """Kernels of lbm_step_observe(n): chunks of 64 steps and a last one of up
+    to 66 that ends with a single step, two reduction kernels each."""
+    total = 0
+    while n > 66:
+        total += (32 if pairs else 64) + 2
+        n -= 64
+    if n:
+        m = (n - 1) // 2 if pairs else 0
+        total += m + (n - 2 * m) + 2
+    return total
+
+
 def traffic_from_profiles(workload="cathode-4096x1024", precision="fp32"):
-    """DRAM bytes per launch of the step kernel from the committed ncu
+    """DRAM bytes per step of the two-step kernel from the committed ncu
     summary of a workload and storage, if one exists for the current kernel."""
-    path = os.path.join(ROOT, "profiles", f"k_step_{workload}-{precision}.json")
+    path = os.path.join(ROOT, "profiles", f"k_step2_{workload}-{precision}.json")
     if os.path.exists(path):
         try:
             j = json.load(open(path))
             if j.get("kernel_source_hash") == kernel_source_hash(precision):
-                return float(j["dram_bytes_per_launch"])
+                return float(j["dram_bytes_per_launch"]) / j["steps_per_launch"]
         except Exception:
             pass
     return None
@@ -252,8 +272,10 @@ def kernel_source_hash(precision="fp32"):
     for name in STEP_SOURCES + (STORAGE_UNIT[precision],):
         h.update(open(os.path.join(csrc, name), "rb").read())
     launch = open(os.path.join(csrc, "lbm_launch.h")).read()
-    shapes = re.search(r"kStepShapes\[kStepVariants\] = \{[^;]*;", launch)
-    h.update(shapes.group(0).encode() if shapes else b"")
+    for pattern in (r"kStepShapes\[kStepVariants\] = \{[^;]*;", r"kStripCols = [^;]*;",
+                    r"pair_blocks_per_sm\([^}]*}"):
+        found = re.search(pattern, launch)
+        h.update(found.group(0).encode() if found else b"")
     return h.hexdigest()[:16]
 
 
@@ -403,7 +425,8 @@ def run_ours(args):
         barrier(pg, dev)
         torch.cuda.synchronize()
         clk.mark()
-        ms, launches = timed_steps(d, K, stream, args.residual_every)
+        spp = steps_per_pass(args.precision, args.rounding)
+        ms, launches = timed_steps(d, K, stream, args.residual_every, spp == 2)
     torch.cuda.synchronize()
     barrier(pg, dev)
     ms_max = max_over_ranks(ms, pg, dev)
@@ -425,7 +448,8 @@ def run_ours(args):
     ms_step = ms_max / K
     value = world * cells * K / (ms_max * 1e-3) / 1e6
     bpc = d.bytes_per_cell()
-    achieved = bpc * cells / (ms_step * 1e-3) / 1e9
+    # a pass moves a step's bytes and takes spp steps
+    achieved = bpc / spp * cells / (ms_step * 1e-3) / 1e9
     peak, peak_kind = measured_peak()
     line = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": K,
@@ -453,8 +477,9 @@ def run_ours(args):
                      "traffic": (traffic_from_profiles(precision=args.precision)
                                  if args.workload == "blocks" and (args.nx, args.ny) == (NX, NY)
                                  else None),
-                     "peak_source": peak_kind, "bytes_per_cell": bpc,
-                     "kernel": "k_step (coupled collide+stream)"},
+                     "peak_source": peak_kind, "bytes_per_cell": bpc, "steps_per_pass": spp,
+                     "kernel": ("k_step2 (two coupled steps per pass)" if spp == 2
+                                else "k_step (coupled collide+stream)")},
         "gpu_launches": launches,
         "step": ("coupled update of every cell (a1-a7) with the per-step current-density and "
                  f"heat reduction copied to the host (a8), and the residual every "
@@ -478,17 +503,17 @@ def run_ours(args):
 def warm_up(d, W):
     """W untimed steps through the calls the timed region makes (observed
     steps and a residual), so that their first-call set-up (observation
-    slots, side stream, step graphs, residual snapshot) happens before the
+    slots, step graphs, residual snapshot) happens before the
     timing starts."""
     i_buf, h_buf = np.zeros(W), np.zeros(W)
     d.step_observe(W, i_buf, h_buf)
     d.residual()
 
 
-def timed_steps(d, K, stream, residual_every):
+def timed_steps(d, K, stream, residual_every, pairs):
     """K steps of the whole hot path, timed with CUDA events on the domain's
     stream: each step's coupled update, its current-density and heat
-    reduction copied to pinned host memory as the step completes
+    reduction copied to pinned host memory chunk by chunk
     (lbm_step_observe), and the steady-state residual every residual_every
     steps.  Returns (ms, kernel launches)."""
     import torch
@@ -496,20 +521,19 @@ def timed_steps(d, K, stream, residual_every):
     h_buf = torch.zeros(K, dtype=torch.float64).pin_memory().numpy()
     e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
     e0.record(stream)
-    done, checks = 0, 0
+    done, launches = 0, 0
     while done < K:
         n = min(residual_every, K - done)
         d.step_observe(n, i_buf[done:done + n], h_buf[done:done + n])
         done += n
+        launches += observed_launches(n, pairs)
         if n == residual_every:
             d.residual()
-            checks += 1
+            launches += 2   # the residual kernel and its block sum
     e1.record(stream)
     e1.synchronize()
     assert np.isfinite(i_buf).all()
-    # per step: the step kernel, the catalyst reduction and its column sum;
-    # per check: the residual kernel and its block sum
-    return e0.elapsed_time(e1), 3 * K + 2 * checks
+    return e0.elapsed_time(e1), launches
 
 
 def sweep_run(cases, args, stream):
@@ -619,7 +643,7 @@ def end_to_end(case, precision, K, stream, interface_mode=0):
     The job runs twice on one domain.  The first run also makes what a
     domain keeps between jobs: the device arrays the material and the fields
     pass through, and the library's work space made at first use (palette
-    build scratch, observation slots and side stream).  The second run, the
+    build scratch, observation slots).  The second run, the
     reported one, repeats every step of the job itself on that domain."""
     import torch
     from paper_2103_01444_gb300.units import cathode_params
@@ -870,7 +894,11 @@ def run_validation(args):
     barrier(pg, dev)
     with ClockSampler(local) as clk:
         ms = d.time_steps(K)
-    launches = K   # one step kernel per step (no reductions in the timed region)
+    # two steps per launch, the last one or two alone (no reductions in the
+    # timed region)
+    spp = steps_per_pass(args.precision)
+    pairs = (K - 1) // 2 if spp == 2 else 0
+    launches = K - pairs
     torch.cuda.synchronize()
     ms_max = max_over_ranks(ms, pg, dev)
     b = d.balances()
@@ -878,7 +906,7 @@ def run_validation(args):
         return
     ms_step = ms_max / K
     bpc = d.bytes_per_cell()
-    achieved = bpc * cells / (ms_step * 1e-3) / 1e9
+    achieved = bpc / spp * cells / (ms_step * 1e-3) / 1e9   # a pass takes spp steps
     peak, peak_kind = measured_peak()
     state = {k: b[k] for k in ("in_T", "out_T", "J", "in_O2")}
     if case["kind"] == "cavity":
@@ -905,9 +933,8 @@ def run_validation(args):
                                  if args.workload == "cavity" and args.precision == "fp32"
                                  and case["nx"] == 2048 else None),
                      "peak_source": peak_kind,
-                     "bytes_per_cell": bpc,
-                     "kernel": "k_step, extended instantiation (" +
-                               ("128 x 2" if variant <= 2 else "64 x 2") + " threads per block)"},
+                     "bytes_per_cell": bpc, "steps_per_pass": spp,
+                     "kernel": ("k_step2" if spp == 2 else "k_step") + ", extended instantiation"},
         "gpu_launches": launches,
         "step": ("coupled update of every cell (a1-a7) with the per-step current-density and "
                  f"heat reduction copied to the host (a8), and the residual every "

@@ -863,9 +863,9 @@ lbm_status lbm_step(lbm_domain *d, int64_t nsteps) {
   lbm_status s = check_ready(d);
   if (s != LBM_OK) return s;
   if (nsteps < 0) return fail(LBM_EINVAL, "nsteps < 0");
-  // long runs replay a graph; the last step or two are launched on their own
+  // long runs replay a graph; the last steps are launched on their own
   int64_t left = nsteps;
-  while (left >= 2 * kGraphSteps || (d->graph[d->cur] && left >= kGraphSteps + 2)) {
+  while (nsteps >= 2 * kGraphSteps && left >= kGraphSteps + 2) {
     if ((s = ensure_graph(d)) != LBM_OK) return s;
     CK(cudaGraphLaunch(d->graph[d->cur], d->stream));
     left -= kGraphSteps;
@@ -1922,7 +1922,7 @@ lbm_status batch_run(lbm_batch *b, int64_t nsteps, bool fixed_parity) {
          std::memcmp(args.data(), b->conc_args.data(), sizeof(KArgs) * n) != 0))
       drop_batch_graph(b);
     int64_t left = nsteps;
-    while (left >= 2 * kBatchGraphSteps || (b->conc_graph && left >= kBatchGraphSteps + 2)) {
+    while (nsteps >= 2 * kBatchGraphSteps && left >= kBatchGraphSteps + 2) {
       if (!b->conc_graph) {
         cudaGraph_t gr = nullptr;
         CK(cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal));
@@ -2009,7 +2009,7 @@ lbm_status batch_run(lbm_batch *b, int64_t nsteps, bool fixed_parity) {
     return LBM_OK;
   }
   int64_t left = nsteps;
-  while (left >= 2 * kBatchGraphSteps || (b->graph && left >= kBatchGraphSteps + 2)) {
+  while (nsteps >= 2 * kBatchGraphSteps && left >= kBatchGraphSteps + 2) {
     if (!b->graph) {
       cudaGraph_t gr = nullptr;
       CK(cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal));

@@ -86,7 +86,7 @@ k_batch_step2(const BatchCaseT<typename Real<S>::type> *__restrict__ cases,
   __syncthreads();
   const BatchCaseT<R> &bc = cases[c];
   const int cur = bc.cur0 ^ parity;
-  two_steps_unit<S, false, false>(
+  two_steps_unit<S, false>(
       (const S *)bc.pop[cur], (S *)bc.pop[cur ^ 1], bc.mask, bc.mid, (const MatCoef<R> *)bc.pal, sa,
       (blockIdx.x - __ldg(block_start + c)) * kPairWarps + (threadIdx.x >> 5), (R *)nullptr, 0);
 }
@@ -567,10 +567,8 @@ cudaError_t allow_step2() {
   if constexpr (sizeof(S) < 8) {
     const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
     const int n = (int)pair_smem_bytes(sizeof(S));
-    cudaError_t e = cudaFuncSetAttribute(k_step2<S, false, false>, attr, n);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_step2<S, false, true>, attr, n);
-    if constexpr (sizeof(S) == 2)
-      if (e == cudaSuccess) e = cudaFuncSetAttribute(k_step2<S, true, false>, attr, n);
+    cudaError_t e = cudaFuncSetAttribute(k_step2<S, false>, attr, n);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_step2<S, true>, attr, n);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_batch_step2<S>, attr, n);
     const int n4 = (int)quad_smem_bytes(sizeof(S));
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_step4<S, false>, attr, n4);

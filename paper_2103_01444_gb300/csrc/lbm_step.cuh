@@ -248,15 +248,16 @@ k_step(const S *__restrict__ src_p, S *__restrict__ dst, const uint8_t *__restri
 // A single step of this lattice is bound by HBM (FP32, 0.95 of the measured
 // copy rate at 4096 x 1024) or by latency and issue (16 bits); a pair moves
 // the same bytes for two steps and is bound by issue and by what is left of
-// the memory latency (FP32: 62% of issue slots, 2.0 of 5.6 warp cycles per
-// issue wait for loads).  One warp alone owns its ring, so no block barrier
+// the memory latency (FP32: 64% of issue slots, 2.0 of 5.5 warp cycles per
+// issue wait for loads, 848 MB of DRAM a pass at 5.1 TB/s; BF16: 78% of issue
+// slots).  One warp alone owns its ring, so no block barrier
 // ties warps in different phases together (with blocks of 128 x 2 cells and
 // __syncthreads: 184 us a step).  The next row's pulls are copied into the
 // stage while both steps of this round run, and a column's material stays in
 // registers.  Per step, two at a time against single steps (tuned shape in
-// 16 bits): 4096 x 1024 FP32 81.3 against 124.5 us, BF16 74.3 against 87;
-// 1024 x 256 FP32 9.7 against 11.5; 200 x 40 FP32 3.6 against 6.8.
-template <typename S, bool SR, bool X>
+// 16 bits): 4096 x 1024 FP32 82.3 against 124.5 us, BF16 70.2 against 87;
+// 1000 x 1000 cavity, FP32, 26 against 37.
+template <typename S, bool X>
 __device__ __forceinline__ void two_steps(const S *__restrict__ src_p, S *__restrict__ dst,
                                           const uint8_t *__restrict__ mask,
                                           const uint16_t *__restrict__ mid,
@@ -272,8 +273,6 @@ __device__ __forceinline__ void two_steps(const S *__restrict__ src_p, S *__rest
   const bool own_x = in_x && lane >= 1 && lane <= kStripCols;
   const Pops<S, kLdg> src{src_p, a.plane, a.nxp};
   const Pops<S, kRing> between{ring, x0};
-  unsigned seed = 0;
-  if constexpr (SR) seed = __ldg(a.seed_ctr);
   R *const jout2 = jout ? jout + jstep : nullptr;
   const int y_top = yb < a.ny ? yb : a.ny - 1;   // the last row the second step pulls from
   // this lane's cell in ring row y1 (row y1 - 1 follows two ring rows on,
@@ -334,9 +333,9 @@ __device__ __forceinline__ void two_steps(const S *__restrict__ src_p, S *__rest
       request_interior(src, a, c2, lane, stage, diag);
       m_next = ld_mask(mask, c2, a, 20);
       e_next = ld_mid(mid, c2, a, 21);
-      finish_cell<S, kLdg, SR, X, false, int>(
+      finish_cell<S, kLdg, false, X, false, int>(
           src, ring, hi, kRingCells, mask, mid, pal, a, c1, x, y1, (uint8_t)m_hi, mc, cell, jout,
-          own_x && y1 >= ya && y1 < yb, seed, RecPtrs<R>{});
+          own_x && y1 >= ya && y1 < yb, 0u, RecPtrs<R>{});
     }
     __syncwarp();
     const int y = y1 - 1;
@@ -347,9 +346,9 @@ __device__ __forceinline__ void two_steps(const S *__restrict__ src_p, S *__rest
       Cell<R> cell;
       load_shared(between, lo, c0, hi, cell);
       material(e_lo);
-      finish_cell<S, kRing, SR, X, false, unsigned>(
+      finish_cell<S, kRing, false, X, false, unsigned>(
           between, dst, c, 0u, mask, mid, pal, a, c, x, y, (uint8_t)m_lo, mc, cell, jout2, true,
-          seed + 1u, RecPtrs<R>{});
+          0u, RecPtrs<R>{});
     }
     __syncwarp();   // the next first step overwrites ring row y1 - 2
     hi = hi >= 2 * kRingCols ? hi - 2 * kRingCols : hi + kRingCols;
@@ -363,7 +362,7 @@ __device__ __forceinline__ void two_steps(const S *__restrict__ src_p, S *__rest
 }
 
 // Unit u of a lattice's strips x row chunks, one per warp.
-template <typename S, bool SR, bool X>
+template <typename S, bool X>
 __device__ __forceinline__ void two_steps_unit(const S *src_p, S *dst, const uint8_t *mask,
                                                const uint16_t *mid,
                                                const MatCoef<typename Real<S>::type> *pal,
@@ -389,16 +388,16 @@ __device__ __forceinline__ void two_steps_unit(const S *src_p, S *dst, const uin
   auto row_at = [&](int w) { return w < 2 * a.ny_cl ? (w + 1) >> 1 : min(w - a.ny_cl, a.ny); };
   const int ya = row_at(chunk * a.pair_rows), yb = row_at((chunk + 1) * a.pair_rows);
   if (ya >= yb) return;
-  two_steps<S, SR, X>(src_p, dst, mask, mid, pal, a, strip, ya, yb, jout, jstep, ring, stage);
+  two_steps<S, X>(src_p, dst, mask, mid, pal, a, strip, ya, yb, jout, jstep, ring, stage);
 }
 
-template <typename S, bool SR, bool X>
+template <typename S, bool X>
 __global__ void __launch_bounds__(32 * kPairWarps, pair_blocks_per_sm(sizeof(S)))
 k_step2(const S *__restrict__ src_p, S *__restrict__ dst, const uint8_t *__restrict__ mask,
         const uint16_t *__restrict__ mid, const MatCoef<typename Real<S>::type> *__restrict__ pal,
         KArgsT<typename Real<S>::type> a, typename Real<S>::type *__restrict__ jout,
         long long jstep) {
-  two_steps_unit<S, SR, X>(src_p, dst, mask, mid, pal, a, blockIdx.x * kPairWarps + (threadIdx.x >> 5),
+  two_steps_unit<S, X>(src_p, dst, mask, mid, pal, a, blockIdx.x * kPairWarps + (threadIdx.x >> 5),
                            jout, jstep);
 }
 
@@ -528,27 +527,18 @@ void launch_step(const void *src, void *dst, const DevGeom &g, const KArgs &a, i
   }
 }
 
-// Two steps: a grid of strips x row chunks (KArgsT.pair_rows).
-template <typename S, bool SR, bool X>
-void launch_step2_v(const void *src, void *dst, const DevGeom &g, const KArgs &a, void *jout,
-                    long long jstep, cudaStream_t st) {
-  using R = typename Real<S>::type;
-  k_step2<S, SR, X><<<pair_blocks(a.nx, a.ny, a.ny_cl, a.pair_rows), 32 * kPairWarps,
-                      pair_smem_bytes(sizeof(S)), st>>>(
-      (const S *)src, (S *)dst, g.mask, g.mid, (const MatCoef<R> *)g.pal, narrow_args<R>(a),
-      (R *)jout, jstep);
-}
+// Two steps, one warp per strip and row chunk.
 template <typename S>
 void launch_step2(const void *src, void *dst, const DevGeom &g, const KArgs &a, void *jout,
                   long long jstep, cudaStream_t st) {
   if constexpr (sizeof(S) < 8) {
-    if (needs_extended(a)) return launch_step2_v<S, false, true>(src, dst, g, a, jout, jstep, st);
-    if constexpr (sizeof(S) == 2)
-      if (a.stochastic) return launch_step2_v<S, true, false>(src, dst, g, a, jout, jstep, st);
-    launch_step2_v<S, false, false>(src, dst, g, a, jout, jstep, st);
+    using R = typename Real<S>::type;
+    auto kern = needs_extended(a) ? k_step2<S, true> : k_step2<S, false>;
+    kern<<<pair_blocks(a.nx, a.ny, a.ny_cl, a.pair_rows), 32 * kPairWarps, pair_smem_bytes(sizeof(S)), st>>>(
+        (const S *)src, (S *)dst, g.mask, g.mid, (const MatCoef<R> *)g.pal, narrow_args<R>(a), (R *)jout,
+        jstep);
   }
 }
-
 template <typename S>
 void launch_step4(const void *src, void *dst, const DevGeom &g, const KArgs &a, void *jout,
                   long long jstep, cudaStream_t st) {
