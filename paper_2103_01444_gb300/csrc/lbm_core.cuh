@@ -293,6 +293,7 @@ template <typename F> struct KArgsT {
   F theta0;                 // Cref_T - T_in
   int stochastic;           // 16-bit step stores: 1 stochastic rounding, 0 nearest even
   const unsigned *seed_ctr; // device step counter seeding the stochastic rounding
+  unsigned seed_off;        // this launch's step beyond the counter
   F hpo;                    // temperature per unit O2 consumed (Eq. 15, 16)
   // Boussinesq buoyancy: force per unit mass (gam_x, gam_y) (T - T_buoy),
   // with T - T_buoy = C_T + buoy_off (C_T the deviation sum of the T lattice)
@@ -332,7 +333,7 @@ template <typename F> __host__ __device__ inline KArgsT<F> narrow_args(const KAr
   }
   r.kA_surf = F(a.kA_surf); r.kA_vol = F(a.kA_vol); r.k_ein = F(a.k_ein); r.k_c1 = F(a.k_c1);
   r.T_in = F(a.T_in); r.theta0 = F(a.theta0); r.hpo = F(a.hpo);
-  r.stochastic = a.stochastic; r.seed_ctr = a.seed_ctr;
+  r.stochastic = a.stochastic; r.seed_ctr = a.seed_ctr; r.seed_off = a.seed_off;
   r.kA_surf_a = F(a.kA_surf_a); r.kA_vol_a = F(a.kA_vol_a);
   r.k_ein_a = F(a.k_ein_a); r.k_c1_a = F(a.k_c1_a);
   return r;

@@ -187,7 +187,7 @@ __device__ __forceinline__ void cell_update(const S *__restrict__ src_p, S *__re
   load_interior<S, R, CG>(src, a, x, y, cell);
   const MatCoef<R> mc = pal[ld_mid(mid, c, a, 21)];
   unsigned seed = 0;
-  if constexpr (SR) seed = __ldg(a.seed_ctr);
+  if constexpr (SR) seed = __ldg(a.seed_ctr) + a.seed_off;
   finish_cell<S, CG, SR, X, REC, long long>(src, dst, c, a.plane, mask, mid, pal, a, c, x, y, m, mc,
                                             cell, jout, true, seed, rp);
 }
