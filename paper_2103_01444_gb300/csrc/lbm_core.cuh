@@ -36,7 +36,8 @@ namespace pemlbm {
 // extent of its buffer.  An access outside it is skipped (a load gives 0, a
 // mask load a solid cell) and the first one of each translation unit is
 // recorded as site << 48 | (index & (2^48 - 1)) for lbm_bounds_check.
-// Nothing traps.  Without the flag every check is the constant true.
+// (Site 7 is no index: the rows that a warp of the two-step kernel asked for
+// and has not taken, 0 when it leaves.)  Nothing traps.  Without the flag every check is the constant true.
 #ifdef PEMLBM_BOUNDS_CHECK
 static __device__ unsigned long long g_bounds_first_bad = 0;
 __device__ __forceinline__ bool in_bounds(long long i, long long n, unsigned site) {

@@ -302,9 +302,11 @@ __device__ __forceinline__ void two_steps(const S *__restrict__ src_p, S *__rest
   }
   const int pf_top = a.pair_ahead ? y_top - a.pair_ahead : -2;   // last row y1 that prefetches
   S diag[4] = {};
+  int asked = 0;   // rows asked for and not taken (only the bounds-checked build looks at it)
   if (in_x) {
     const unsigned c = ya > 0 ? c1 : c1 + a.nxp;   // the first row taken
     request_interior(src, a, c, lane, stage, diag);
+    asked = 1;
     m_hi = ld_mask(mask, c, a, 20);
     e_hi = ld_mid(mid, c, a, 21);
   }
@@ -325,14 +327,20 @@ __device__ __forceinline__ void two_steps(const S *__restrict__ src_p, S *__rest
     const bool first = in_x && y1 >= 0 && y1 <= y_top;
     if (first) {   // first step of row y1
       Cell<R> cell;
+      in_bounds(asked - 1, 1, 7);   // the row to take was asked for, once
+      asked -= 1;
       take_interior<S, R>(lane, stage, diag, cell);
       material(e_hi);
-      // the next row is on its way during both steps (past the last row, the
-      // last one again: nothing takes it)
-      const unsigned c2 = c1 + (y1 < y_top ? a.nxp : 0);
-      request_interior(src, a, c2, lane, stage, diag);
-      m_next = ld_mask(mask, c2, a, 20);
-      e_next = ld_mid(mid, c2, a, 21);
+      // the next row is on its way during both steps; none is asked for past
+      // the last, so that every copy into the stage has been waited for when
+      // the warp leaves its shared memory to another block
+      if (y1 < y_top) {
+        const unsigned c2 = c1 + a.nxp;
+        request_interior(src, a, c2, lane, stage, diag);
+        asked += 1;
+        m_next = ld_mask(mask, c2, a, 20);
+        e_next = ld_mid(mid, c2, a, 21);
+      }
       finish_cell<S, kLdg, false, X, false, int>(
           src, ring, hi, kRingCells, mask, mid, pal, a, c1, x, y1, (uint8_t)m_hi, mc, cell, jout,
           own_x && y1 >= ya && y1 < yb, 0u, RecPtrs<R>{});
@@ -359,6 +367,7 @@ __device__ __forceinline__ void two_steps(const S *__restrict__ src_p, S *__rest
       e_hi = e_next;
     }
   }
+  in_bounds(asked, 1, 7);   // no copy may still be on its way
 }
 
 // Unit u of a lattice's strips x row chunks, one per warp.
