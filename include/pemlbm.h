@@ -208,7 +208,11 @@ lbm_status lbm_reset(lbm_domain *d);
 /* Advances nsteps coupled steps (Eq. 1, 10 with the Sec. 4 boundary links):
  * stream with boundary links -> macroscopic values (Eq. 8, 11) ->
  * collisions -> catalyst sources.  Asynchronous on the domain's stream;
- * long runs are replayed from a captured CUDA graph. */
+ * runs of 128 steps or more are replayed from a captured CUDA graph.
+ * Shorter calls only launch kernels, and may be captured into a graph of the
+ * caller's on the domain's stream: its replays march on where nsteps is even
+ * (the two population buffers swap at every odd number of steps), and they do
+ * not advance the domain's step counter. */
 lbm_status lbm_step(lbm_domain *d, int64_t nsteps);
 
 /* Reaction of the last step (Sec. 5 outputs): mean current density over the
