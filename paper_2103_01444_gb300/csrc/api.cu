@@ -1746,20 +1746,20 @@ struct lbm_batch {
   std::vector<cudaEvent_t> ev;      // one per domain, for stream ordering
   cudaEvent_t ev_batch = nullptr, ev0 = nullptr, ev1 = nullptr;
   // schedule 3: one stream ("lane") per case, each case's steps a chain of
-  // single-domain launches; the chains run concurrently, replayed from one
-  // graph captured for the cases' current buffers (conc_cur)
+  // single-domain launches; the chains run concurrently, replayed from a
+  // graph captured for the cases' current buffers (one of two, conc_bufs)
   std::vector<cudaStream_t> lanes;
   std::vector<cudaEvent_t> lane_done;
   cudaEvent_t ev_fork = nullptr;
-  cudaGraphExec_t conc_graph = nullptr;
-  std::vector<int> conc_cur;
+  cudaGraphExec_t conc_graph[2] = {nullptr, nullptr};
+  GraphSlots conc_bufs;
   std::vector<int> flips;           // per case: whether the last run ended in the other buffer
   // schedule 0 in steps of two (every case can_pair): blocks of the two-step
   // kernel, numbered case after case
   bool pairs = false;
   int *dpair = nullptr;             // device prefix sums [ncases + 1]
   int pair_blocks = 0, pair_rows = 0;
-  std::vector<KArgs> conc_args;     // the arguments the graph's launches carry
+  std::vector<KArgs> conc_args;     // the arguments the graphs' launches carry
 };
 
 namespace {
@@ -1771,9 +1771,10 @@ void drop_batch_graph(lbm_batch *b) {
     cudaGraphExecDestroy(b->graph);
     b->graph = nullptr;
   }
-  if (b->conc_graph) {
-    cudaGraphExecDestroy(b->conc_graph);
-    b->conc_graph = nullptr;
+  for (int k = 0; k < 2; ++k) {
+    if (b->conc_graph[k]) cudaGraphExecDestroy(b->conc_graph[k]);
+    b->conc_graph[k] = nullptr;
+    b->conc_bufs.clear(k);
   }
 }
 
@@ -1917,15 +1918,16 @@ lbm_status batch_run(lbm_batch *b, int64_t nsteps, bool fixed_parity) {
       cur[c] = b->doms[c]->cur;
       args[c] = make_args(b->doms[c]);
     }
-    // the graph bakes in each case's buffers and arguments: recapture when
-    // a case was stepped alone or its parameters changed
-    if (b->conc_graph &&
-        (cur != b->conc_cur ||
-         std::memcmp(args.data(), b->conc_args.data(), sizeof(KArgs) * n) != 0))
+    // a graph bakes in each case's buffers and arguments: none is valid after
+    // a change of parameters, and other buffers (a case stepped alone, a run
+    // that ended in the other ones) have a graph of their own
+    if (b->conc_args.size() == args.size() &&
+        std::memcmp(args.data(), b->conc_args.data(), sizeof(KArgs) * n) != 0)
       drop_batch_graph(b);
     int64_t left = nsteps;
     while (nsteps >= 2 * kBatchGraphSteps && left >= kBatchGraphSteps + 2) {
-      if (!b->conc_graph) {
+      int slot = b->conc_bufs.find(cur);
+      if (slot < 0) {
         cudaGraph_t gr = nullptr;
         CK(cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal));
         lbm_status s = batch_lanes(b, kBatchGraphSteps, false, true);
@@ -1935,13 +1937,16 @@ lbm_status batch_run(lbm_batch *b, int64_t nsteps, bool fixed_parity) {
           return s;
         }
         if (e != cudaSuccess) return fail(LBM_ECUDA, "lane graph capture: %s", cudaGetErrorString(e));
-        e = cudaGraphInstantiate(&b->conc_graph, gr, 0);
+        cudaGraphExec_t ge = nullptr;
+        e = cudaGraphInstantiate(&ge, gr, 0);
         cudaGraphDestroy(gr);
         if (e != cudaSuccess) return fail(LBM_ECUDA, "lane graph instantiate: %s", cudaGetErrorString(e));
-        b->conc_cur = cur;
+        slot = b->conc_bufs.take(cur);
+        if (b->conc_graph[slot]) cudaGraphExecDestroy(b->conc_graph[slot]);
+        b->conc_graph[slot] = ge;
         b->conc_args = args;
       }
-      CK(cudaGraphLaunch(b->conc_graph, b->stream));   // even count: parities return
+      CK(cudaGraphLaunch(b->conc_graph[slot], b->stream));   // even count: parities return
       left -= kBatchGraphSteps;
     }
     return batch_lanes(b, left, false, false);

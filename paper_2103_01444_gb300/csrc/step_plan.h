@@ -2,6 +2,7 @@
 // only, without CUDA headers.
 #pragma once
 #include <cstdint>
+#include <vector>
 
 namespace pemlbm {
 
@@ -36,5 +37,27 @@ inline StepPlan plan_steps(bool quad, bool pair, int64_t n, bool open, bool keep
   }
   return p;
 }
+
+// Which of the two graphs that a batch keeps was captured for given buffers
+// (one per case).  A run of an even number of steps leaves each case where it
+// was or in its other buffer, the same at every call of that count, so calls
+// alternate between two sets of buffers at most.
+struct GraphSlots {
+  std::vector<int> bufs[2];   // empty: no graph in that slot
+  int newest = 1;
+  // the slot of the graph for these buffers, -1 for none
+  int find(const std::vector<int> &b) const {
+    for (int k = 0; k < 2; ++k)
+      if (!bufs[k].empty() && bufs[k] == b) return k;
+    return -1;
+  }
+  // the slot that a new graph for these buffers takes: the older one
+  int take(const std::vector<int> &b) {
+    newest ^= 1;
+    bufs[newest] = b;
+    return newest;
+  }
+  void clear(int slot) { bufs[slot].clear(); }
+};
 
 }  // namespace pemlbm

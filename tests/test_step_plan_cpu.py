@@ -55,3 +55,42 @@ def test_an_even_number_of_steps_keeps_the_buffer(plans):
         # the graphs of 64 steps return to their buffer by themselves
         if go_on and n == 64:
             assert (quads + pairs + singles) % 2 == 0
+
+
+SLOTS = r"""
+#include <cstdio>
+#include <vector>
+#include "step_plan.h"
+// calls of `n` steps of a batch of two pairable cases and one that is stepped
+// one by one, as lbm_batch_step makes them: graphs captured
+int captures(int n, int calls) {
+  pemlbm::GraphSlots slots;
+  std::vector<int> cur{0, 1, 0};
+  int made = 0;
+  for (int c = 0; c < calls; ++c) {
+    int left = n;
+    while (n >= 128 && left >= 66) {
+      if (slots.find(cur) < 0) {
+        slots.take(cur);
+        ++made;
+      }
+      left -= 64;
+    }
+    for (int k = 0; k < 3; ++k) cur[k] ^= pemlbm::plan_steps(false, k < 2, left, false, false).launches() & 1;
+  }
+  return made;
+}
+int main() {
+  for (int n = 128; n <= 600; ++n) std::printf("%d %d\n", n, captures(n, 40));
+}
+"""
+
+
+def test_repeated_batch_calls_capture_two_graphs_at_most(tmp_path):
+    (tmp_path / "slots.cc").write_text(SLOTS)
+    subprocess.check_call(["g++", "-std=c++17", "-I", CSRC, str(tmp_path / "slots.cc"), "-o",
+                           str(tmp_path / "slots")])
+    out = subprocess.check_output([str(tmp_path / "slots")], text=True)
+    made = dict(tuple(map(int, line.split())) for line in out.splitlines())
+    assert len(made) == 473 and max(made.values()) <= 2
+    assert made[130] == 1 and made[128] == 2   # 130 steps come back to their buffers, 128 swap them
