@@ -343,7 +343,11 @@ lbm_status lbm_bytes_per_cell(lbm_domain *d, double *bytes);
  * are the same either way, so the result does not depend on the limit.
  * Memory: the stored segments' records, plus, when some segment is
  * recomputed, one population state per recomputed segment and two
- * segments' records.  The gradient of the
+ * segments' records; and the reverse workspace (four sets of adjoint
+ * populations in the arithmetic type, two states, six fields), which stays
+ * with the domain for its next lbm_grad or lbm_vjp while the workspaces of
+ * all domains are below 1/64 of the device's memory, until the domain is
+ * destroyed or its limit is set to 0 (lbm_set_grad_memory).  The gradient of the
  * Fickian interface mode treats each scalar's b (that of its largest
  * diffusivity) as fixed.  dphi, dK, dD_O2 are [ny][nx] doubles (NULL to
  * skip): host memory with on_device = 0, device memory written on the
@@ -359,9 +363,11 @@ lbm_status lbm_grad(lbm_domain *d, int32_t objective, int64_t nsteps, int32_t se
 
 /* Device memory lbm_grad may hold for the reverse records of stored
  * segments (bytes): -1 (the default) for what is free less the reserve, 0
- * to recompute every segment from its checkpoint.  The setting is the
- * domain's and applies to its later lbm_grad calls.  EINVAL for a null
- * domain or bytes < -1. */
+ * to recompute every segment from its checkpoint, and to hold nothing
+ * between calls: the reverse workspace that earlier calls left with the
+ * domain is released (after the work on its stream), and later ones leave
+ * none.  The setting is the domain's and applies to its later lbm_grad and
+ * lbm_vjp calls.  EINVAL for a null domain or bytes < -1. */
 lbm_status lbm_set_grad_memory(lbm_domain *d, int64_t bytes);
 
 /* Self-check of the device code's indexing (no counterpart in the paper; it

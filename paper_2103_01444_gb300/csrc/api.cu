@@ -7,6 +7,7 @@
 #include <nvtx3/nvToolsExt.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -160,8 +161,7 @@ struct lbm_domain {
   bool halo_lo = false, halo_hi = false;
   std::vector<uint8_t> hsolid;                 // the whole lattice's solids (slabs)
   cudaEvent_t ev_halo = nullptr;
-  // reverse workspace of lbm_grad and lbm_vjp, kept between calls when small
-  // (adj_work)
+  // reverse workspace of lbm_grad and lbm_vjp, kept between calls (AdjLease)
   void *adj = nullptr;
   void (*adj_free)(void *) = nullptr;
 };
@@ -1209,18 +1209,29 @@ struct DevBuf {
   }
 };
 
+// Bytes of reverse workspaces that stay with their domains between calls, of
+// all domains of the process.
+std::atomic<size_t> g_adj_kept{0};
+
 // Reverse workspace of one domain.
 struct AdjWork {
   DevBuf lam[2], O[2], V[2], gphi, gK, gD, gU, tphi, tK, tD, cells, pushed, slot, fs[2];
-  size_t bytes = 0;                             // of the lattice-sized buffers
+  size_t bytes = 0;                             // of all its buffers
+  size_t kept = 0;                              // what it counts for in g_adj_kept
   int n_edge = 0, n_own = 0;
   size_t rsize = 4;                             // bytes of the arithmetic type
   cudaStream_t side = nullptr;                  // edge-cell branch of each step
   cudaEvent_t fork = nullptr, join = nullptr;
   ~AdjWork() {
+    g_adj_kept -= kept;
     if (fork) cudaEventDestroy(fork);
     if (join) cudaEventDestroy(join);
     if (side) cudaStreamDestroy(side);
+  }
+  lbm_status take(DevBuf &b, size_t n) {
+    lbm_status s = b.alloc(n);
+    if (s == LBM_OK) bytes += n;
+    return s;
   }
   lbm_status alloc(lbm_domain *d) {
     const size_t r = fp64(d) ? 8 : 4, planes = 24 * (size_t)d->plane;
@@ -1232,20 +1243,18 @@ struct AdjWork {
       return fail(LBM_ECUDA, "stream or event creation for the adjoint failed");
     }
     for (auto *b : {&lam[0], &lam[1], &O[0], &O[1]})
-      if ((s = b->alloc(planes * r)) != LBM_OK) return s;
+      if ((s = take(*b, planes * r)) != LBM_OK) return s;
     for (auto *b : {&V[0], &V[1]})   // [outlet, inlet][down, up][10][ny]
-      if ((s = b->alloc(40 * (size_t)d->ny * r)) != LBM_OK) return s;
+      if ((s = take(*b, 40 * (size_t)d->ny * r)) != LBM_OK) return s;
     // forward states, with the guard of a domain's buffers
     const size_t sbytes = (24 * (size_t)d->plane + d->nxp + 64) * d->esize;
     for (auto &b : fs)
-      if ((s = b.alloc(sbytes)) != LBM_OK) return s;
-    bytes = 4 * planes * r + 2 * sbytes + 3 * (r + sizeof(double)) * (size_t)d->plane +
-            sizeof(int) * (size_t)d->plane;
+      if ((s = take(b, sbytes)) != LBM_OK) return s;
     for (auto *b : {&gphi, &gK, &gD})
-      if ((s = b->alloc(r * d->plane)) != LBM_OK) return s;
+      if ((s = take(*b, r * d->plane)) != LBM_OK) return s;
     for (auto *b : {&tphi, &tK, &tD})
-      if ((s = b->alloc(sizeof(double) * d->plane)) != LBM_OK) return s;
-    if ((s = gU.alloc(sizeof(double))) != LBM_OK) return s;
+      if ((s = take(*b, sizeof(double) * d->plane)) != LBM_OK) return s;
+    if ((s = take(gU, sizeof(double))) != LBM_OK) return s;
     // cell lists: fluid cells with edge bits, then fluid catalyst cells of
     // the volumetric mode without them (both use their own state)
     std::vector<uint8_t> m((size_t)d->plane);
@@ -1276,7 +1285,7 @@ struct AdjWork {
     // listed index of every cell (reverse records of own states), -1 for others
     std::vector<int> slots((size_t)d->plane, -1);
     for (size_t t = 0; t < list.size(); ++t) slots[(size_t)list[t]] = (int)t;
-    if ((s = slot.alloc(sizeof(int) * slots.size())) != LBM_OK) return s;
+    if ((s = take(slot, sizeof(int) * slots.size())) != LBM_OK) return s;
     CK(cudaMemcpyAsync(slot.p, slots.data(), sizeof(int) * slots.size(), cudaMemcpyHostToDevice,
                        d->stream));
     CK(cudaStreamSynchronize(d->stream));
@@ -1299,12 +1308,12 @@ struct AdjWork {
       bits[t] = b;
     }
     if (n_own > 0) {
-      if ((s = cells.alloc(sizeof(long long) * list.size())) != LBM_OK) return s;
+      if ((s = take(cells, sizeof(long long) * list.size())) != LBM_OK) return s;
       CK(cudaMemcpyAsync(cells.p, list.data(), sizeof(long long) * list.size(),
                          cudaMemcpyHostToDevice, d->stream));
     }
     if (n_edge > 0) {
-      if ((s = pushed.alloc(sizeof(uint32_t) * bits.size())) != LBM_OK) return s;
+      if ((s = take(pushed, sizeof(uint32_t) * bits.size())) != LBM_OK) return s;
       CK(cudaMemcpyAsync(pushed.p, bits.data(), sizeof(uint32_t) * bits.size(),
                          cudaMemcpyHostToDevice, d->stream));
     }
@@ -1356,22 +1365,21 @@ struct AdjWork {
 
 // The reverse workspace of a domain for one call.  Its allocations, the cell
 // lists built on the host and the matching frees took 1.9 ms of every call
-// (1024 x 256), so it stays with the domain until that is destroyed where it
-// is below 1/64 of the device's memory, and is released after the call beyond
-// that.
+// (1024 x 256), so it stays with the domain for its next call while the
+// workspaces kept by all domains are below 1/64 of the device's memory, and is
+// released after the call beyond that, or where the domain's limit of
+// lbm_set_grad_memory is 0.
 struct AdjLease {
   lbm_domain *d = nullptr;
   AdjWork *w = nullptr;
-  bool keep = false;
   ~AdjLease() {
-    if (!w || keep) return;
+    if (!w || w->kept) return;
     cudaStreamSynchronize(d->stream);
     delete w;
     d->adj = nullptr;
   }
   lbm_status take(lbm_domain *dom) {
     d = dom;
-    size_t free_b = 0, total_b = 0;
     if (!d->adj) {
       w = new AdjWork();
       lbm_status s = w->alloc(d);
@@ -1380,8 +1388,15 @@ struct AdjLease {
       d->adj_free = [](void *p) { delete (AdjWork *)p; };
     }
     w = (AdjWork *)d->adj;
-    CK(cudaMemGetInfo(&free_b, &total_b));
-    keep = w->bytes <= total_b / 64;
+    if (!w->kept && d->grad_mem_limit != 0) {
+      size_t free_b = 0, total_b = 0;
+      CK(cudaMemGetInfo(&free_b, &total_b));
+      w->kept = w->bytes;
+      if ((g_adj_kept += w->kept) > total_b / 64) {
+        g_adj_kept -= w->kept;
+        w->kept = 0;
+      }
+    }
     return w->begin(d);
   }
 };
@@ -1721,6 +1736,11 @@ lbm_status lbm_set_grad_memory(lbm_domain *d, int64_t bytes) {
   if (!d) return fail(LBM_EINVAL, "null domain");
   if (bytes < -1) return fail(LBM_EINVAL, "bytes must be -1 (automatic) or >= 0");
   d->grad_mem_limit = bytes;
+  if (bytes == 0 && d->adj) {   // the workspace of earlier calls
+    CK(cudaStreamSynchronize(d->stream));
+    d->adj_free(d->adj);
+    d->adj = nullptr;
+  }
   return LBM_OK;
 }
 

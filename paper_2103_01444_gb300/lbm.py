@@ -339,7 +339,7 @@ class Domain:
     def set_grad_memory(self, nbytes: int):
         """Device bytes grad() may keep reverse records in: -1 for what is
         free (the default), 0 to recompute every segment from its
-        checkpoint."""
+        checkpoint and to hold no workspace between calls."""
         _check(self.L.lbm_set_grad_memory(self.h, int(nbytes)))
 
     def vjp(self, lam_next):
