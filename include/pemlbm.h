@@ -344,10 +344,11 @@ lbm_status lbm_bytes_per_cell(lbm_domain *d, double *bytes);
  * Memory: the stored segments' records, plus, when some segment is
  * recomputed, one population state per recomputed segment and two
  * segments' records; and the reverse workspace (four sets of adjoint
- * populations in the arithmetic type, two states, six fields), which stays
- * with the domain for its next lbm_grad or lbm_vjp while the workspaces of
- * all domains are below 1/64 of the device's memory, until the domain is
- * destroyed or its limit is set to 0 (lbm_set_grad_memory).  The gradient of the
+ * populations in the arithmetic type, two states (one in lbm_vjp), six
+ * fields), which stays with the domain for its next lbm_grad or lbm_vjp
+ * while the workspaces of all domains are below 1/64 of the device's
+ * memory, until the domain is destroyed or its limit is set to 0
+ * (lbm_set_grad_memory).  The gradient of the
  * Fickian interface mode treats each scalar's b (that of its largest
  * diffusivity) as fixed.  dphi, dK, dD_O2 are [ny][nx] doubles (NULL to
  * skip): host memory with on_device = 0, device memory written on the

@@ -1233,6 +1233,15 @@ struct AdjWork {
     if (s == LBM_OK) bytes += n;
     return s;
   }
+  // The first n forward states, with the guard of a domain's buffers.
+  lbm_status states(const lbm_domain *d, int n) {
+    for (int k = 0; k < n; ++k)
+      if (!fs[k].p) {
+        lbm_status s = take(fs[k], (24 * (size_t)d->plane + d->nxp + 64) * d->esize);
+        if (s != LBM_OK) return s;
+      }
+    return LBM_OK;
+  }
   lbm_status alloc(lbm_domain *d) {
     const size_t r = fp64(d) ? 8 : 4, planes = 24 * (size_t)d->plane;
     lbm_status s;
@@ -1246,10 +1255,6 @@ struct AdjWork {
       if ((s = take(*b, planes * r)) != LBM_OK) return s;
     for (auto *b : {&V[0], &V[1]})   // [outlet, inlet][down, up][10][ny]
       if ((s = take(*b, 40 * (size_t)d->ny * r)) != LBM_OK) return s;
-    // forward states, with the guard of a domain's buffers
-    const size_t sbytes = (24 * (size_t)d->plane + d->nxp + 64) * d->esize;
-    for (auto &b : fs)
-      if ((s = take(b, sbytes)) != LBM_OK) return s;
     for (auto *b : {&gphi, &gK, &gD})
       if ((s = take(*b, r * d->plane)) != LBM_OK) return s;
     for (auto *b : {&tphi, &tK, &tD})
@@ -1378,7 +1383,7 @@ struct AdjLease {
     delete w;
     d->adj = nullptr;
   }
-  lbm_status take(lbm_domain *dom) {
+  lbm_status take(lbm_domain *dom, int states) {
     d = dom;
     if (!d->adj) {
       w = new AdjWork();
@@ -1388,14 +1393,15 @@ struct AdjLease {
       d->adj_free = [](void *p) { delete (AdjWork *)p; };
     }
     w = (AdjWork *)d->adj;
-    if (!w->kept && d->grad_mem_limit != 0) {
+    g_adj_kept -= w->kept;
+    w->kept = 0;
+    lbm_status s = w->states(d, states);
+    if (s != LBM_OK) return s;
+    if (d->grad_mem_limit != 0) {
       size_t free_b = 0, total_b = 0;
       CK(cudaMemGetInfo(&free_b, &total_b));
-      w->kept = w->bytes;
-      if ((g_adj_kept += w->kept) > total_b / 64) {
-        g_adj_kept -= w->kept;
-        w->kept = 0;
-      }
+      if ((g_adj_kept += w->bytes) <= total_b / 64) w->kept = w->bytes;
+      else g_adj_kept -= w->bytes;
     }
     return w->begin(d);
   }
@@ -1514,14 +1520,13 @@ lbm_status lbm_vjp(lbm_domain *d, const double *lam_next, double *lam_prev, doub
   if (d->desc.rounding != 0) return fail(LBM_EINVAL, "the adjoint needs round-to-nearest storage");
   if ((s = adjoint_covers(d)) != LBM_OK) return s;
   AdjLease lease;
-  if ((s = lease.take(d)) != LBM_OK) return s;
+  if ((s = lease.take(d, 1)) != LBM_OK) return s;
   AdjWork &w = *lease.w;
   if ((s = lam_upload(d, lam_next, w.lam[0].p)) != LBM_OK) return s;
-  // the step's reverse records (its new state is not kept)
-  DevBuf rec, next;
+  // the step's reverse records (its new state is not used)
+  DevBuf rec;
   if ((s = rec.alloc(w.rec_bytes(d))) != LBM_OK) return s;
-  if ((s = next.alloc((24 * (size_t)d->plane + d->nxp + 64) * d->esize)) != LBM_OK) return s;
-  step_with_records(d, d->pop[d->cur], next.p, w.recs(d, rec.p), d->stream);
+  step_with_records(d, d->pop[d->cur], w.fs[0].p, w.recs(d, rec.p), d->stream);
   reverse_step(d, w, 0, w.recs(d, rec.p), -1, true);
   finish_lambda(d, w, 1);
   CK(cudaGetLastError());
@@ -1550,7 +1555,7 @@ lbm_status lbm_grad(lbm_domain *d, int32_t objective, int64_t nsteps, int32_t se
   const int64_t nseg = (nrec + seg - 1) / seg;   // segment k: R^{k seg + 1} .. R^{min((k+1) seg, nrec)}
   const size_t sbytes = (24 * (size_t)d->plane + d->nxp + 64) * d->esize;   // guard as in the domain
   AdjLease lease;
-  if ((s = lease.take(d)) != LBM_OK) return s;
+  if ((s = lease.take(d, 2)) != LBM_OK) return s;
   AdjWork &w = *lease.w;
   DevBuf(&fs)[2] = w.fs;   // forward states
   const size_t rbytes = w.rec_bytes(d), segbytes = rbytes * (size_t)seg;

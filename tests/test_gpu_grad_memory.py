@@ -45,6 +45,27 @@ def test_the_workspace_is_released_on_request():
         np.testing.assert_array_equal(g0[k], g[k])
 
 
+def test_a_transposed_step_takes_one_state():
+    """lbm_vjp takes (and leaves) one population state, not the two that a
+    gradient steps between and a third one."""
+    nx, ny = 1024, 256
+    d = domain(nx, ny, "fp32")
+    lam = np.random.default_rng(0).standard_normal((24, ny, nx))
+    d.vjp(lam)                           # (loads the kernels)
+    d.set_grad_memory(0)
+    before = free_bytes()
+    d.set_grad_memory(-1)
+    d.vjp(lam)
+    held = before - free_bytes()
+    state, cells = 96 * nx * ny, nx * ny
+    # four sets of adjoint populations, six fields, the listed index, one state
+    assert held < 4 * state + 40 * cells + 1.5 * state, held / state
+    J = d.grad(0, 6)[0]                  # a gradient takes its second state
+    assert before - free_bytes() > 4 * state + 40 * cells + 1.5 * state
+    d.set_grad_memory(0)
+    assert d.grad(0, 6)[0] == J
+
+
 def test_kept_workspaces_are_bounded_over_all_domains():
     import torch
     total = torch.cuda.mem_get_info()[1]
