@@ -229,9 +229,14 @@ lbm_status lbm_current_density(lbm_domain *d, double *i_avg_A_cm2, double *heat_
  * not both).  A step's reacting cells leave the O2 they consume beside their
  * populations; chunks of 64 steps are replayed from CUDA graphs, and each
  * chunk's FP64 sums are copied to the host, which converts them while the
- * next chunk runs.  Synchronises the stream before returning.  EINVAL for nsteps < 0
- * or two NULL arrays; ENOMEM if the observation slots cannot be
- * allocated. */
+ * next chunk runs.  The first call allocates those values, which stay with the
+ * domain: 66 x reacting rows x nx of the arithmetic type.  Where that is more
+ * than a quarter of the two population buffers (and than 64 MB), or does not
+ * fit, chunks are shorter (32, 16 or 8 steps), and where not even 10 x rows x
+ * nx values fit, every step's reaction is recomputed from the state before it
+ * instead.  The results are the same.  Synchronises the stream before
+ * returning.  EINVAL for nsteps < 0 or two NULL arrays; ENOMEM if the slots of
+ * the sums (4 KB) cannot be allocated. */
 lbm_status lbm_step_observe(lbm_domain *d, int64_t nsteps, double *i_avg_A_cm2,
                             double *heat_W_cm2);
 

@@ -59,8 +59,8 @@ struct NvtxRange {
 
 // Host-side fault injection for tests of the ENOMEM paths: with
 // PEMLBM_FAIL_ALLOC=n in the environment, the n-th allocation the library
-// makes after the variable last changed fails as if memory were exhausted.
-// Nothing reaches the device.
+// makes after the variable last changed fails as if memory were exhausted
+// ("n+": that one and all later ones).  Nothing reaches the device.
 bool inject_alloc_failure() {
   static std::mutex mu;
   static std::string last;
@@ -73,7 +73,8 @@ bool inject_alloc_failure() {
     count = 0;
   }
   if (cur.empty()) return false;
-  return ++count == std::atol(cur.c_str());
+  const long n = std::atol(cur.c_str());
+  return ++count == n || (cur.back() == '+' && count > n);
 }
 template <typename T> cudaError_t dmalloc(T **p, size_t bytes) {
   if (inject_alloc_failure()) {
@@ -92,6 +93,7 @@ template <typename T> cudaError_t hmalloc(T **p, size_t bytes) {
 
 constexpr int kGraphSteps = 64;   // even: a replay returns to the same buffer
 constexpr int kObsSlots = kGraphSteps + 2;   // steps of the longest observed chunk
+constexpr int kObsLeast = 8;      // graph steps of the shortest one (an even number of fours)
 constexpr int kMaxPalette = 65535;
 
 size_t elem_size(int prec) {
@@ -147,10 +149,11 @@ struct lbm_domain {
   cudaGraphExec_t graph[2] = {nullptr, nullptr};
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
   // observed stepping: the O2 each reacting cell consumes in every step of a
-  // chunk [kObsSlots][reacting rows][nx] (arithmetic precision), its column
-  // sums, the per-step (J, heat) sums in device slots [2][kObsSlots][2], and
-  // pinned host slots of the same shape; one graph per (starting buffer,
-  // slot half)
+  // chunk [obs_steps + 2][reacting rows][nx] (arithmetic precision) and its
+  // column sums, where there was room for them; the per-step (J, heat) sums in
+  // device slots [2][kObsSlots][2], and pinned host slots of the same shape;
+  // one graph of obs_steps steps per (starting buffer, slot half)
+  int obs_steps = kGraphSteps;
   void *jcells = nullptr;
   double *jcol = nullptr, *dobs = nullptr, *hobs = nullptr;
   cudaGraphExec_t obs_graph[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};
@@ -372,17 +375,30 @@ lbm_status ensure_graph(lbm_domain *d) {
   return LBM_OK;
 }
 
-// Observed steps: n steps (n <= kObsSlots) that also write the O2 every
+// Observed steps: n steps (n <= obs_steps + 2) that also write the O2 every
 // reacting cell consumes, [step][reacting row][nx], then the FP64 sums of
-// every step and their copy to the pinned host slots of `half`.
+// every step and their copy to the pinned host slots of `half`.  Without room
+// for the cells' values each step is taken alone and its reaction recomputed
+// from the state it left behind, as lbm_current_density does.
 lbm_status launch_observed(lbm_domain *d, int64_t n, bool open, int half) {
-  const int64_t rows = d->desc.reaction_mode == 1 ? d->desc.ny_cl : 1;
-  lbm_status s = launch_steps(d, n, open, d->jcells, rows * d->nx);
-  if (s != LBM_OK) return s;
-  const KArgs a = make_args(d);
   const size_t slot = (size_t)half * kObsSlots * 2;
-  launch_sum_reaction(d->jcells, fp64(d), d->nx, (int)rows, (int)n, a.hpo, d->jcol, d->dobs + slot,
-                      d->stream);
+  const KArgs a = make_args(d);
+  lbm_status s;
+  if (d->jcells) {
+    const int64_t rows = d->desc.reaction_mode == 1 ? d->desc.ny_cl : 1;
+    if ((s = launch_steps(d, n, open, d->jcells, rows * d->nx)) != LBM_OK) return s;
+    launch_sum_reaction(d->jcells, fp64(d), d->nx, (int)rows, (int)n, a.hpo, d->jcol, d->dobs + slot,
+                        d->stream);
+  } else {
+    for (int64_t k = 0; k < n; ++k) {
+      if ((s = launch_steps(d, 1)) != LBM_OK) return s;
+      dispatch(d->desc.precision, [&](auto *tag) {
+        using S = std::remove_pointer_t<decltype(tag)>;
+        launch_catalyst<S>(d->pop[d->cur ^ 1], geom(d), a, 1.0, nullptr, d->colsum,
+                           d->dobs + slot + 2 * k, d->ddone, d->stream);
+      });
+    }
+  }
   CK(cudaMemcpyAsync(d->hobs + slot, d->dobs + slot, (size_t)n * 2 * sizeof(double),
                      cudaMemcpyDeviceToHost, d->stream));
   CK(cudaGetLastError());
@@ -395,7 +411,7 @@ lbm_status ensure_obs_graph(lbm_domain *d, int half) {
   const int start = d->cur;
   cudaGraph_t gr = nullptr;
   CK(cudaStreamBeginCapture(d->stream, cudaStreamCaptureModeThreadLocal));
-  lbm_status s = launch_observed(d, kGraphSteps, true, half);
+  lbm_status s = launch_observed(d, d->obs_steps, true, half);
   cudaError_t e = cudaStreamEndCapture(d->stream, &gr);
   d->cur = start;
   if (s != LBM_OK) {
@@ -409,30 +425,47 @@ lbm_status ensure_obs_graph(lbm_domain *d, int half) {
   return LBM_OK;
 }
 
-// First-use work space of observed stepping, all or nothing.
+// First-use work space of observed stepping.  The cells' values of a chunk of
+// 64 steps are small beside the state on a thin catalyst (4096 x 1024, 51
+// rows: 55 MB of 805), but a lattice that is all catalyst would take more than
+// its populations; so chunks are halved, down to kObsLeast steps, while the
+// values take more than a quarter of the two states (and more than 64 MB) or
+// cannot be allocated, and left out where not even the shortest chunk's fit.
 lbm_status ensure_observation(lbm_domain *d) {
   if (d->dobs) return LBM_OK;
   const size_t bytes = 2 * kObsSlots * 2 * sizeof(double);
   const size_t rows = d->desc.reaction_mode == 1 ? d->desc.ny_cl : 1;
-  const size_t jbytes = (size_t)kObsSlots * rows * d->nx * (fp64(d) ? 8 : 4);
-  double *dobs = nullptr, *hobs = nullptr, *jcol = nullptr;
-  void *jcells = nullptr;
+  const size_t jstep = rows * d->nx * (fp64(d) ? 8 : 4), cstep = sizeof(double) * 2 * d->nx;
+  const size_t most = std::max<size_t>(12 * (size_t)d->plane * d->esize, (size_t)64 << 20);
+  double *dobs = nullptr, *hobs = nullptr;
   cudaEvent_t done[2] = {nullptr, nullptr};
   if (dmalloc(&dobs, bytes) != cudaSuccess || hmalloc(&hobs, bytes) != cudaSuccess ||
-      dmalloc(&jcol, sizeof(double) * 2 * kObsSlots * d->nx) != cudaSuccess ||
-      dmalloc(&jcells, jbytes) != cudaSuccess ||
       cudaEventCreateWithFlags(&done[0], cudaEventDisableTiming) != cudaSuccess ||
-      cudaEventCreateWithFlags(&done[1], cudaEventDisableTiming) != cudaSuccess ||
-      // cells that never react (solids) keep their zeros
-      cudaMemsetAsync(jcells, 0, jbytes, d->stream) != cudaSuccess) {
-    for (void *p : {(void *)dobs, (void *)jcol, jcells})
-      if (p) cudaFree(p);
+      cudaEventCreateWithFlags(&done[1], cudaEventDisableTiming) != cudaSuccess) {
+    if (dobs) cudaFree(dobs);
     if (hobs) cudaFreeHost(hobs);
     for (cudaEvent_t e : done)
       if (e) cudaEventDestroy(e);
     cudaGetLastError();
-    return fail(LBM_ENOMEM, "observation slots (%.1f MB)", jbytes / 1e6);
+    return fail(LBM_ENOMEM, "observation slots");
   }
+  double *jcol = nullptr;
+  void *jcells = nullptr;
+  int steps = kGraphSteps;
+  while (steps > kObsLeast && (steps + 2) * jstep > most) steps /= 2;
+  for (; steps >= kObsLeast; steps /= 2) {
+    const size_t slots = steps + 2;
+    // cells that never react (solids) keep their zeros
+    if (dmalloc(&jcol, slots * cstep) == cudaSuccess && dmalloc(&jcells, slots * jstep) == cudaSuccess &&
+        cudaMemsetAsync(jcells, 0, slots * jstep, d->stream) == cudaSuccess)
+      break;
+    for (void *p : {(void *)jcol, jcells})
+      if (p) cudaFree(p);
+    jcol = nullptr;
+    jcells = nullptr;
+    cudaGetLastError();
+  }
+  d->obs_steps = jcells ? steps : kGraphSteps;
   d->dobs = dobs;
   d->hobs = hobs;
   d->jcol = jcol;
@@ -935,8 +968,8 @@ lbm_status lbm_step_observe(lbm_domain *d, int64_t nsteps, double *i_avg, double
   int64_t done = 0, prev_first = -1, prev_n = 0;
   int half = 0;
   while (done < nsteps) {
-    const bool last = nsteps - done <= kObsSlots;
-    const int64_t n = last ? nsteps - done : kGraphSteps;
+    const bool last = nsteps - done <= d->obs_steps + 2;
+    const int64_t n = last ? nsteps - done : d->obs_steps;
     if (!last) {
       if ((s = ensure_obs_graph(d, half)) != LBM_OK) return s;
       CK(cudaGraphLaunch(d->obs_graph[d->cur][half], d->stream));   // cur unchanged
