@@ -222,24 +222,50 @@ class ClockSampler:
                 "samples": len(sm)}
 
 
-def steps_per_pass(precision, rounding="nearest"):
-    """Steps that one pass over the populations takes on these lattices: the
-    library runs two per launch (k_step2) except in FP64 and with stochastic
-    rounding."""
-    return 1 if precision == "fp64" or rounding != "nearest" else 2
+def steps_at_once(case, precision, rounding="nearest"):
+    """How the library launches the steps of a whole lattice: 4 at a time on
+    small ones (at most 1216 of k_step4's 26 x 10 cell blocks), 2 (k_step2), or
+    1 in FP64, with stochastic rounding and in periodic lattices."""
+    if precision == "fp64" or rounding != "nearest" or case.get("periodic_x"):
+        return 1
+    return 4 if -(-case["nx"] // 26) * -(-case["ny"] // 10) <= 1216 else 2
 
 
-def observed_launches(n, pairs):
-    """Kernels of lbm_step_observe(n): chunks of 64 steps and a last one of up
-    to 66 that ends with a single step, two reduction kernels each."""
-    total = 0
-    while n > 66:
-        total += (32 if pairs else 64) + 2
-        n -= 64
-    if n:
-        m = (n - 1) // 2 if pairs else 0
-        total += m + (n - 2 * m) + 2
+def run_launches(n, most, goes_on=False):
+    """Step kernels of a run of n steps, at most `most` at a time: fours, pairs,
+    then single steps, with a single step at the end unless the run goes on."""
+    left = n - (0 if goes_on or n == 0 else 1)
+    total = n - left
+    for k in (4, 2, 1):
+        if k <= most:
+            total += left // k
+            left %= k
     return total
+
+
+def step_launches(n, most):
+    """Step kernels of lbm_step(n): replays of a graph of 64 steps from 128
+    steps on, then a run of up to 65."""
+    total, left = 0, n
+    while n >= 128 and left >= 66:
+        total += run_launches(64, most, True)
+        left -= 64
+    return total + run_launches(left, most)
+
+
+def observed_launches(n, most, stochastic=False):
+    """Kernels of lbm_step_observe(n): chunks of 64 steps and a last one of up
+    to 66, each with two reduction kernels (and the step counter of stochastic
+    rounding)."""
+    extra, total = 2 + bool(stochastic), 0
+    while n > 66:
+        total += run_launches(64, most, True) + extra
+        n -= 64
+    return total + (run_launches(n, most) + extra if n else 0)
+
+
+STEP_KERNEL = {1: "k_step (coupled collide+stream)", 2: "k_step2 (two coupled steps per pass)",
+               4: "k_step4 (four coupled steps per pass)"}
 
 
 def traffic_from_profiles(workload="cathode-4096x1024", precision="fp32"):
@@ -425,8 +451,9 @@ def run_ours(args):
         barrier(pg, dev)
         torch.cuda.synchronize()
         clk.mark()
-        spp = steps_per_pass(args.precision, args.rounding)
-        ms, launches = timed_steps(d, K, stream, args.residual_every, spp == 2)
+        spp = steps_at_once(case, args.precision, args.rounding)
+        ms, launches = timed_steps(d, K, stream, args.residual_every, spp,
+                                   args.rounding != "nearest")
     torch.cuda.synchronize()
     barrier(pg, dev)
     ms_max = max_over_ranks(ms, pg, dev)
@@ -478,8 +505,7 @@ def run_ours(args):
                                  if args.workload == "blocks" and (args.nx, args.ny) == (NX, NY)
                                  else None),
                      "peak_source": peak_kind, "bytes_per_cell": bpc, "steps_per_pass": spp,
-                     "kernel": ("k_step2 (two coupled steps per pass)" if spp == 2
-                                else "k_step (coupled collide+stream)")},
+                     "kernel": STEP_KERNEL[spp]},
         "gpu_launches": launches,
         "step": ("coupled update of every cell (a1-a7) with the per-step current-density and "
                  f"heat reduction copied to the host (a8), and the residual every "
@@ -510,7 +536,7 @@ def warm_up(d, W):
     d.residual()
 
 
-def timed_steps(d, K, stream, residual_every, pairs):
+def timed_steps(d, K, stream, residual_every, most, stochastic=False):
     """K steps of the whole hot path, timed with CUDA events on the domain's
     stream: each step's coupled update, its current-density and heat
     reduction copied to pinned host memory chunk by chunk
@@ -526,7 +552,7 @@ def timed_steps(d, K, stream, residual_every, pairs):
         n = min(residual_every, K - done)
         d.step_observe(n, i_buf[done:done + n], h_buf[done:done + n])
         done += n
-        launches += observed_launches(n, pairs)
+        launches += observed_launches(n, most, stochastic)
         if n == residual_every:
             d.residual()
             launches += 2   # the residual kernel and its block sum
@@ -894,11 +920,9 @@ def run_validation(args):
     barrier(pg, dev)
     with ClockSampler(local) as clk:
         ms = d.time_steps(K)
-    # two steps per launch, the last one or two alone (no reductions in the
-    # timed region)
-    spp = steps_per_pass(args.precision)
-    pairs = (K - 1) // 2 if spp == 2 else 0
-    launches = K - pairs
+    # (no reductions in the timed region)
+    spp = steps_at_once(case, args.precision)
+    launches = step_launches(K, spp)
     torch.cuda.synchronize()
     ms_max = max_over_ranks(ms, pg, dev)
     b = d.balances()
@@ -934,7 +958,7 @@ def run_validation(args):
                                  and case["nx"] == 2048 else None),
                      "peak_source": peak_kind,
                      "bytes_per_cell": bpc, "steps_per_pass": spp,
-                     "kernel": ("k_step2" if spp == 2 else "k_step") + ", extended instantiation"},
+                     "kernel": STEP_KERNEL[spp] + ", extended instantiation"},
         "gpu_launches": launches,
         "step": ("coupled update of every cell (a1-a7) with the per-step current-density and "
                  f"heat reduction copied to the host (a8), and the residual every "
