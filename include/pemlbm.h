@@ -300,17 +300,20 @@ lbm_status lbm_get_step(lbm_domain *d, int64_t *steps);
 lbm_status lbm_save_state(lbm_domain *d, void *buf, size_t *bytes);
 lbm_status lbm_load_state(lbm_domain *d, const void *buf, size_t bytes);
 
-/* Average device time per launch of the coupled-step kernel over the last
- * lbm_step call that was timed with lbm_time_steps (ms), for roofline
- * reporting: runs nsteps steps bracketed by CUDA events on the domain's
- * stream and returns the elapsed device time. */
+/* Runs nsteps steps as lbm_step does, bracketed by CUDA events on the domain's
+ * stream, and returns the elapsed device time (ms). */
 lbm_status lbm_time_steps(lbm_domain *d, int64_t nsteps, double *elapsed_ms);
 
-/* Launch shapes of the step kernel (cells per block along x and y, and the
- * minimum resident blocks per SM asked of the register allocator).
- * lbm_tune, called between lbm_reset and the first step, times every shape
- * over trial_steps launches of the same step (the state is left as reset
- * left it), keeps the fastest and returns its index and time per step (ms).
+/* Launch shapes of the kernel that takes a single step (cells per block along
+ * x and y, and the minimum resident blocks per SM asked of the register
+ * allocator).  lbm_tune, called between lbm_reset and the first step, times
+ * every shape over trial_steps launches of the same step (the state is left
+ * as reset left it), keeps the fastest and returns its index and the time of
+ * such a launch (ms).  Whole lattices that are not periodic, stored in FP32 or
+ * in 16 bits with round to nearest, take their steps two or four per launch,
+ * in kernels that have one shape: there the chosen shape serves the last one
+ * or two steps of a call, and a step of a longer run takes less than the time
+ * returned (lbm_time_steps measures it).
  * ESTATE after the first step.  lbm_set_variant selects one explicitly
  * (0 <= variant < 8; EINVAL otherwise).  All shapes give bit-identical
  * results.  Untuned, FP64 domains use variant 0 (32 x 4 cells; FP64 has its
@@ -409,7 +412,8 @@ lbm_status lbm_vjp(lbm_domain *d, const double *lam_next, double *lam_prev, doub
  * stream, ordered after and before the other domains' streams by events.
  * Schedules (lbm_batch_set_schedule):
  *   0  one launch per step covering every case's tiles (launch shape
- *      `variant` of lbm_set_variant), long runs replayed from a CUDA graph;
+ *      `variant` of lbm_set_variant), or per two steps where every case may
+ *      step in pairs (lbm_tune), long runs replayed from a CUDA graph;
  *   1  one persistent cooperative launch for all steps: co-resident blocks
  *      loop over the tiles and meet at a grid barrier between steps; each
  *      barrier wait gives up after spin_limit polls (<= 0 keeps the current
@@ -418,12 +422,16 @@ lbm_status lbm_vjp(lbm_domain *d, const double *lam_next, double *lam_prev, doub
  *   2  one launch per case and step, no graph (the unbatched reference);
  *   3  one stream per case, each case's steps a chain of single-domain
  *      launches (shape `variant`), the chains running concurrently; long
- *      runs replayed from one graph, captured again when a case was stepped
- *      on its own or its arguments changed.
+ *      runs replayed from a graph, one for each of the last two sets of
+ *      buffers that the cases started from, captured again when a case's
+ *      arguments changed.
  * All schedules give bit-identical states.  lbm_batch_tune, called between
- * lbm_reset and the first step of every case, times schedules 0 and 3 with
- * every launch shape and schedule 1 over trial_steps repetitions of the
- * first step, keeps the fastest and leaves the states as reset left them. */
+ * lbm_reset and the first step of every case, times schedules 0 and 3 over
+ * trial_steps repetitions of the first two steps, with every launch shape, or
+ * with shape 7 alone where every case takes its steps in pairs (lbm_tune), and
+ * schedule 1 over trial_steps repetitions of the first step; it keeps the one
+ * with the shortest time per step, returns that time (ms), and leaves the
+ * states as reset left them. */
 typedef struct lbm_batch lbm_batch; /* opaque */
 lbm_status lbm_create_batch(lbm_domain *const *domains, int32_t ncases, lbm_batch **out);
 lbm_status lbm_destroy_batch(lbm_batch *b);

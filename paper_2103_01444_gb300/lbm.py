@@ -392,8 +392,9 @@ class Domain:
         _check(self.L.lbm_load_state(self.h, blob, len(blob)))
 
     def tune(self, trial_steps: int = 20):
-        """Times every launch shape of the step kernel (after reset, before the
-        first step) and keeps the fastest; returns (variant, ms per step)."""
+        """Times every launch shape of the single-step kernel (after reset,
+        before the first step) and keeps the fastest; returns (variant, ms of
+        a single step).  Steps taken two or four per launch take less."""
         v, ms = C.c_int32(), C.c_double()
         _check(self.L.lbm_tune(self.h, int(trial_steps), C.byref(v), C.byref(ms)))
         return v.value, ms.value
