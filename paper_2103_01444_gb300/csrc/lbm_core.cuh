@@ -802,6 +802,14 @@ __device__ __forceinline__ void take_interior(int lane, const unsigned char *sta
 template <int CG, typename S, typename R>
 __device__ __forceinline__ void load_shared(const Pops<S, CG> &src, int lo, int c0, int hi, Cell<R> &c) {
   constexpr int P = CG == kRing ? kRingCells : kTileCells;
+#ifdef PEMLBM_BOUNDS_CHECK
+  // the sources are these three cells and the ones beside them
+  for (const int k : {lo, c0, hi})
+    if (!in_bounds(k - 1, P, CG == kRing ? 5 : 6) || !in_bounds(k + 1, P, CG == kRing ? 5 : 6)) {
+      c = Cell<R>{};
+      return;
+    }
+#endif
   const int from[5] = {c0, c0 - 1, lo, c0 + 1, hi};
 #pragma unroll
   for (int i = 0; i < 5; ++i) {
