@@ -223,12 +223,20 @@ class ClockSampler:
 
 
 def steps_at_once(case, precision, rounding="nearest"):
-    """How the library launches the steps of a whole lattice: 4 at a time on
-    small ones (at most 1216 of k_step4's 26 x 10 cell blocks), 2 (k_step2), or
-    1 in FP64, with stochastic rounding and in periodic lattices."""
+    """How many steps a launch takes in a run on a whole lattice, as the library
+    chooses (steps_at_once in csrc/step_plan.h): 4 (k_step4) on small lattices,
+    2 (k_step2) where two states exceed the L2 cache, else 1; always 1 in FP64,
+    with stochastic rounding and in periodic lattices."""
     if precision == "fp64" or rounding != "nearest" or case.get("periodic_x"):
         return 1
-    return 4 if -(-case["nx"] // 26) * -(-case["ny"] // 10) <= 1216 else 2
+    nx, ny, esize = case["nx"], case["ny"], d_esize(precision)
+    if -(-nx // 26) * -(-ny // 10) <= 456:
+        return 4
+    if 48 * (-(-nx // 64) * 64) * ny * esize <= 96e6:
+        return 1
+    if esize == 4:
+        return 2 if nx >= 180 else 1
+    return 2 if nx >= 1024 and 4 * case["ny_cl"] <= ny else 1
 
 
 def run_launches(n, most, goes_on=False):

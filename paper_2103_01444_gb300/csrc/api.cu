@@ -22,7 +22,6 @@
 #include "../../include/pemlbm.h"
 #include "lbm_core.cuh"
 #include "lbm_launch.h"
-#include "step_plan.h"
 
 using namespace pemlbm;
 
@@ -203,7 +202,7 @@ KArgs make_args(const lbm_domain *d) {
   // rows that the two-step kernel asks the L2 cache for ahead of use: only
   // where the two states do not stay in it from pass to pass (1024 x 256 FP32:
   // 9.6 us a step without, 10.2 with; 4096 x 1024: 85.8 without, 81.3 with)
-  a.pair_ahead = 48.0 * d->plane * d->esize > 96e6 ? 3 : 0;
+  a.pair_ahead = 48.0 * d->plane * d->esize > kStatesInL2 ? 3 : 0;
   for (int k = 0; k < 3; ++k)
     for (int s = 0; s < 3; ++s) a.Cwall[k][s] = p.C_wall[k][s];
   a.u_in_avg = p.inlet_mode == 0 ? p.u_in_avg : 0.0;
@@ -286,19 +285,15 @@ void drop_graphs(lbm_domain *d) {
 // storage types whose step is bound by memory (the FP64 step is bound by its
 // arithmetic), with planes that 32-bit byte offsets reach.  A slab needs its
 // halo between the steps.  Stochastic rounding issues too much for the pair to
-// gain (8192 x 2048 grains, FP16: 510 us a step in pairs, 497 one by one).
+// gain (8192 x 2048 grains, FP16: 478 us a step in pairs, 433 one by one).
+// Whether a run takes them so is steps_at_once's choice.
 bool can_pair(const lbm_domain *d) {
   return !fp64(d) && d->desc.rounding == 0 && !d->desc.periodic_x && d->nx == d->nxg &&
          d->plane * 4 * (long long)d->esize < (1LL << 32);
 }
 
-// Whether four steps may run as one launch (k_step4): where pairs may, on
-// lattices of at most eight of its blocks per SM.  us a step in pairs and in
-// fours, FP32: 200 x 40 (32 blocks) 3.5, 2.0; 640 x 160 (400) 5.9, 4.1; 1024 x
-// 256 (1040) 10.0, 8.5; 1300 x 320 (1600) 12.6, 12.8.
-bool can_quad(const lbm_domain *d) {
-  const long long blocks = (long long)((d->nx + kQuadCols - 1) / kQuadCols) * ((d->ny + kQuadRows - 1) / kQuadRows);
-  return can_pair(d) && blocks <= 8 * 152;
+int at_once(const lbm_domain *d) {
+  return can_pair(d) ? steps_at_once(d->nx, d->ny, d->nxp, d->desc.ny_cl, (int)d->esize) : 1;
 }
 
 // The launches of a plan on stream st, from buffer cur of d on; the j-th
@@ -348,7 +343,8 @@ void note_capture(lbm_domain *d, cudaStream_t st) {
 
 lbm_status launch_steps(lbm_domain *d, int64_t n, bool open = false, void *jout = nullptr,
                         int64_t jstep = 0) {
-  const StepPlan plan = plan_steps(can_quad(d), can_pair(d), n, open, d->captured);
+  const int most = at_once(d);
+  const StepPlan plan = plan_steps(most == 4, most >= 2, n, open, d->captured);
   lbm_status s = launch_plan(d, make_args(d), plan, d->cur, d->variant, jout, jstep, d->stream);
   if (s == LBM_OK) d->cur ^= (int)(plan.launches() & 1);
   return s;

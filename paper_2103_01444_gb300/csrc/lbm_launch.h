@@ -4,6 +4,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "step_plan.h"
+
 namespace pemlbm {
 
 template <typename F> struct KArgsT;
@@ -33,8 +35,8 @@ constexpr size_t pair_smem_bytes(size_t esize) {
 }
 constexpr int pair_blocks_per_sm(size_t esize) { return esize == 4 ? 8 : 10; }
 // Shape of the four-step kernel: blocks of 16 warps, a row of 32 columns each,
-// that finish kQuadCols x kQuadRows cells; two tiles of shared memory.
-constexpr int kQuadCols = 26, kQuadRows = 10;
+// that finish kQuadCols x kQuadRows cells (step_plan.h); two tiles of shared
+// memory.
 constexpr size_t quad_smem_bytes(size_t esize) { return 2 * 24 * 512 * esize; }
 // Weighted rows of a unit's chunk for one lattice or the cases of a batch, and
 // a lattice's blocks.

@@ -254,9 +254,9 @@ k_step(const S *__restrict__ src_p, S *__restrict__ dst, const uint8_t *__restri
 // ties warps in different phases together (with blocks of 128 x 2 cells and
 // __syncthreads: 184 us a step).  The next row's pulls are copied into the
 // stage while both steps of this round run, and a column's material stays in
-// registers.  Per step, two at a time against single steps (tuned shape in
-// 16 bits): 4096 x 1024 FP32 82.3 against 124.5 us, BF16 70.2 against 87;
-// 1000 x 1000 cavity, FP32, 26 against 37.
+// registers.  Per step, two at a time against single steps: 4096 x 1024 FP32 83
+// against 121 us, BF16 70 against 78; 1000 x 1000 cavity, FP32, 26 against 32
+// (steps_at_once: where they pay).
 template <typename S, bool X>
 __device__ __forceinline__ void two_steps(const S *__restrict__ src_p, S *__restrict__ dst,
                                           const uint8_t *__restrict__ mask,
@@ -418,7 +418,7 @@ k_step2(const S *__restrict__ src_p, S *__restrict__ dst, const uint8_t *__restr
 // instructions (about 1.6 us) and of a launch; here four steps pay for one
 // launch, one load from the L2 cache and four times that latency, where
 // k_step2's warps walk four rows in turn for two steps.  200 x 40, FP32: 2.0
-// us a step against 3.5 in pairs and 6.9 one by one (can_quad: where the
+// us a step against 3.5 in pairs and 3.1 one by one (steps_at_once: where the
 // repeated work outweighs it).
 template <typename S, bool X>
 __global__ void __launch_bounds__(32 * kTileWarps, 1)

@@ -10,9 +10,10 @@ pytestmark = pytest.mark.gpu
 
 
 def lattices():
-    # in fours; in pairs (too many blocks for fours); always one by one
-    return [("fp32", W.small_cathode(200, 40, 1)), ("fp32", W.cathode_blocks(2610, 130)),
-            ("bf16", W.cathode_blocks(2610, 130)), ("fp64", W.small_cathode(96, 30, 0))]
+    # in fours; in pairs (two states larger than the cache); one by one
+    return [("fp32", W.small_cathode(200, 40, 1)), ("fp32", W.cathode_blocks(1024, 500, Re=3.0)),
+            ("bf16", W.cathode_blocks(2048, 500, Re=3.0)), ("fp32", W.cathode_blocks(900, 225, Re=3.0)),
+            ("fp64", W.small_cathode(96, 30, 0))]
 
 
 @pytest.mark.parametrize("n", [4, 6, 8, 10, 12, 20])

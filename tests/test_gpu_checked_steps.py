@@ -27,7 +27,7 @@ def check(what):
 bounds_check()                                   # clears the record
 # one strip and several, one chunk of rows and many, catalyst rows, walls
 cases = [W.small_cathode(30, 24, 0), W.small_cathode(31, 25, 1), W.small_cathode(152, 64, 0, grains=True),
-         W.small_cathode(331, 97, 1), W.cathode_blocks(2610, 130), W.natural_convection_cavity(95)]
+         W.small_cathode(331, 97, 1), W.cathode_blocks(2048, 500, Re=3.0), W.natural_convection_cavity(95)]
 for precision in ("fp32", "bf16", "fp16"):
     for case in cases:
         label = f"{case['nx']}x{case['ny']} {precision}"
