@@ -310,10 +310,11 @@ lbm_status lbm_time_steps(lbm_domain *d, int64_t nsteps, double *elapsed_ms);
  * every shape over trial_steps launches of the same step (the state is left
  * as reset left it), keeps the fastest and returns its index and the time of
  * such a launch (ms).  Whole lattices that are not periodic, stored in FP32 or
- * in 16 bits with round to nearest, take their steps two or four per launch,
- * in kernels that have one shape: there the chosen shape serves the last one
- * or two steps of a call, and a step of a longer run takes less than the time
- * returned (lbm_time_steps measures it).
+ * in 16 bits with round to nearest, may step in pairs, or four at a time on
+ * small ones, in kernels that have one shape; lbm_step chooses by size and
+ * storage.  There the chosen shape serves the last one to three steps of a
+ * call, and a step of a longer run takes less than the time returned
+ * (lbm_time_steps measures it).
  * ESTATE after the first step.  lbm_set_variant selects one explicitly
  * (0 <= variant < 8; EINVAL otherwise).  All shapes give bit-identical
  * results.  Untuned, FP64 domains use variant 0 (32 x 4 cells; FP64 has its
@@ -428,7 +429,7 @@ lbm_status lbm_vjp(lbm_domain *d, const double *lam_next, double *lam_prev, doub
  * All schedules give bit-identical states.  lbm_batch_tune, called between
  * lbm_reset and the first step of every case, times schedules 0 and 3 over
  * trial_steps repetitions of the first two steps, with every launch shape, or
- * with shape 7 alone where every case takes its steps in pairs (lbm_tune), and
+ * with shape 7 alone where every case may step in pairs (lbm_tune), and
  * schedule 1 over trial_steps repetitions of the first step; it keeps the one
  * with the shortest time per step, returns that time (ms), and leaves the
  * states as reset left them. */

@@ -201,7 +201,7 @@ KArgs make_args(const lbm_domain *d) {
   a.pair_rows = d->pair_rows;
   // rows that the two-step kernel asks the L2 cache for ahead of use: only
   // where the two states do not stay in it from pass to pass (1024 x 256 FP32:
-  // 9.6 us a step without, 10.2 with; 4096 x 1024: 85.8 without, 81.3 with)
+  // 9.7 us a step without, 9.6 with; 4096 x 1024: 90.8 without, 83.3 with)
   a.pair_ahead = 48.0 * d->plane * d->esize > kStatesInL2 ? 3 : 0;
   for (int k = 0; k < 3; ++k)
     for (int s = 0; s < 3; ++s) a.Cwall[k][s] = p.C_wall[k][s];

@@ -92,9 +92,10 @@ void launch_seed_advance(unsigned *ctr, unsigned n, cudaStream_t st) {
 // uneven (the end columns cost more), so with more of them than fit the GPU
 // at once the time is their total over the slots plus most of one unit, and
 // with fewer twice an even unit's.  Measured, FP32, us a step: 4096 x 1024 at
-// 8 / 12 / 16 / 24 / 32 / 48 rows 88 / 83 / 81 / 85 / 94 / 122 (the rule
-// takes 16); 1024 x 256 at 1 / 2 / 3 / 4 / 8 rows 11.4 / 9.6 / 9.7 / 10.2 /
-// 14.9 (3); 200 x 40 at 1 / 2 / 8 rows 3.6 / 4.7 / 11.9 (1).
+// 8 / 12 / 14 / 16 / 24 / 32 / 48 rows 87 / 84 / 83 / 81 / 82 / 90 / 116 (the
+// rule takes 14), BF16 73 / 71 / 70 / 70 / 72 / 77 / 100; 1024 x 256 at 1 / 2 /
+// 3 / 4 / 8 rows 11.7 / 9.9 / 9.7 / 10.1 / 14.5 (3); 200 x 40 at 1 / 2 / 8 rows
+// 3.5 / 4.7 / 11.4 (1).
 static long long pair_units(int nx, int ny, int ny_cl, int rows) {
   return (long long)((nx + kStripCols - 1) / kStripCols) * ((ny + ny_cl + rows - 1) / rows);
 }

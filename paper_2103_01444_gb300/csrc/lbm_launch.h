@@ -24,7 +24,7 @@ constexpr StepShape kStepShapes[kStepVariants] = {
 // Shape of the two-step kernel: a warp per strip of kStripCols columns (its
 // first step covers one column more on either side) and chunk of rows.  Its
 // shared memory holds a ring of three rows of 24 populations per lane and
-// the stage of the row on its way (Stage).  FP32: 16 warps per SM at 120
+// the stage of the row on its way (Stage).  FP32: 16 warps per SM at 118
 // registers (limited by shared memory); 16 bits: 20 warps at 96.  With more
 // warps the kernel spills, and beside the rings there is little L1 cache left
 // to hold what it spills (4096 x 1024, us a step: FP32 16 / 18 warps 81 / 88,
